@@ -735,31 +735,108 @@ __global__ void __launch_bounds__(kSX * kSY) prolong_pair_kernel(const float* __
 // coarsest level of at most 4^3: one V-cycle from zero, 2n + 8 red-black
 // sweeps on the coarsest level; as the coarse-grid correction of the outer
 // cycle it needs no more (on the 256^3 benchmark the refinement takes the
-// same number of steps as with two cycles and 2n^2 + 16 sweeps).  Otherwise
-// (a single level, e.g. an odd grid, or a larger coarsest level): two
-// V-cycles, 2n^2 + 16 sweeps on the coarsest level.
+// same number of steps as with two cycles and 2n^2 + 16 sweeps).  Any other
+// coarsest level (an odd grid of 5^3 to 15^3, or a lone level) is solved
+// directly in the cosine basis.  Relaxing it to rounding instead took 2n^2 +
+// 16 sweeps, two cycles of them on a lone level: 932 sweeps at 15^3, four
+// barriers each pair, bound by barrier latency in the one block.  The six
+// transforms give the same correction to FP32 rounding (chi unchanged to
+// ~1e-10 of its spread).  Forward solve at 120^3 (coarsest 15^3): 34.1 -> 1.0
+// ms; at 88^3 (11^3): 9.5 -> 0.8 ms.
 constexpr int kSmallCap = 4096 + 512 + 64 + 27 + 8;
-constexpr int kSmallCycles = 1;     // V-cycles of the coarse-grid solve
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallQ = 15 * 15;    // cosine basis of the largest coarsest level
 
-__device__ void small_rbgs(float* x, const float* b, int n, int color) {
-  const int N = n * n * n;
-  for (int t = threadIdx.x; t < N; t += blockDim.x) {
-    const int i = t % n, j = (t / n) % n, k = t / (n * n);
-    if (((i + j + k) & 1) != color) continue;
-    float acc = 0.f;
-    int cnt = 0;
-    if (i > 0) { acc += x[t - 1]; ++cnt; }
-    if (i < n - 1) { acc += x[t + 1]; ++cnt; }
-    if (j > 0) { acc += x[t - n]; ++cnt; }
-    if (j < n - 1) { acc += x[t + n]; ++cnt; }
-    if (k > 0) { acc += x[t - n * n]; ++cnt; }
-    if (k < n - 1) { acc += x[t + n * n]; ++cnt; }
-    x[t] = cnt ? (acc - b[t]) / (float)cnt : 0.f;
+// `sweeps` red-black sweeps, colour `first` first.  A thread owns up to two
+// pairs of x neighbours (one cell of each colour; found once, not per sweep)
+// and updates the one of the half-sweep's colour.
+__device__ void small_rbgs(float* x, const float* b, int n, int sweeps, int first) {
+  const int hw = (n + 1) >> 1, items = n * n * hw;
+  int t0[2], par[2], im[2];
+  unsigned edge[2];   // bits 0-3: y - 1, y + 1, z - 1, z + 1 inside
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int q = threadIdx.x + a * kSmallThreads;
+    const int row = q / hw, m = q - row * hw;
+    const int k = row / n, j = row - k * n;
+    t0[a] = row * n;
+    im[a] = q < items ? 2 * m : n;      // no cell: i is past the row for both colours
+    par[a] = (j + k) & 1;
+    edge[a] = (j > 0 ? 1u : 0u) | (j < n - 1 ? 2u : 0u) | (k > 0 ? 4u : 0u) | (k < n - 1 ? 8u : 0u);
+  }
+  for (int h = 0; h < 2 * sweeps; ++h) {
+    const int color = first ^ (h & 1);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const int i = im[a] + (par[a] ^ color);
+      if (i >= n) continue;
+      const int t = t0[a] + i;
+      float acc = 0.f;
+      int cnt = 0;
+      if (i > 0) { acc += x[t - 1]; ++cnt; }
+      if (i < n - 1) { acc += x[t + 1]; ++cnt; }
+      if (edge[a] & 1u) { acc += x[t - n]; ++cnt; }
+      if (edge[a] & 2u) { acc += x[t + n]; ++cnt; }
+      if (edge[a] & 4u) { acc += x[t - n * n]; ++cnt; }
+      if (edge[a] & 8u) { acc += x[t + n * n]; ++cnt; }
+      x[t] = cnt ? (acc - b[t]) / (float)cnt : 0.f;
+    }
+    __syncthreads();
+  }
+}
+
+// Orthonormal cosine basis q[k][i] (DCT-II) of a small level.
+__device__ void small_basis(float* q, int n) {
+  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
+    const int k = t / n, i = t - k * n;
+    const int m = (k * (2 * i + 1)) % (4 * n);   // the angle's whole turns dropped exactly
+    q[t] = sqrtf((k ? 2.f : 1.f) / (float)n) * cospif((float)m / (2.f * (float)n));
   }
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(1024) small_vcycle_kernel(float* __restrict__ xg, const float* __restrict__ bg,
+// out = the transform (or its inverse) of in along the axis of stride st.
+__device__ void small_transform(const float* in, float* out, int n, int st, const float* q, bool inverse) {
+  const int N = n * n * n;
+  for (int t = threadIdx.x; t < N; t += blockDim.x) {
+    const int c = (t / st) % n;
+    const float* p = in + (t - c * st);
+    float acc = 0.f;
+    for (int r = 0; r < n; ++r) acc = fmaf(inverse ? q[r * n + c] : q[c * n + r], p[r * st], acc);
+    out[t] = acc;
+  }
+  __syncthreads();
+}
+
+// x = the zero-mean solution of L x = b (q1: of L' x = b) on a small level; b
+// is overwritten.
+__device__ void small_direct(float* x, float* b, int n, const float* q, bool q1) {
+  small_transform(b, x, n, 1, q, false);
+  small_transform(x, b, n, n, q, false);
+  small_transform(b, x, n, n * n, q, false);
+  for (int t = threadIdx.x; t < n * n * n; t += blockDim.x) {
+    const int k[3] = {t % n, (t / n) % n, t / (n * n)};
+    float s[3];
+    for (int a = 0; a < 3; ++a) {
+      const float v = sinpif((float)k[a] / (2.f * (float)n));
+      s[a] = 4.f * v * v;
+    }
+    float lam = -(s[0] + s[1] + s[2]);
+    if (q1) {
+      const float m0 = 1.f - s[0] * (1.f / 6.f), m1 = 1.f - s[1] * (1.f / 6.f), m2 = 1.f - s[2] * (1.f / 6.f);
+      lam = -(float)kQ1Scale * (s[0] * m1 * m2 + m0 * (s[1] * m2 + m1 * s[2]));
+    }
+    x[t] = t ? x[t] / lam : 0.f;
+  }
+  __syncthreads();
+  small_transform(x, b, n, n * n, q, true);
+  small_transform(b, x, n, n, q, true);
+  small_transform(x, b, n, 1, q, true);
+  for (int t = threadIdx.x; t < n * n * n; t += blockDim.x) x[t] = b[t];
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kSmallThreads) small_vcycle_kernel(float* __restrict__ xg, const float* __restrict__ bg,
                                                             const float* __restrict__ shift, int n0,
                                                             const int* __restrict__ gate) {
   if (*gate) return;
@@ -767,6 +844,7 @@ __global__ void __launch_bounds__(1024) small_vcycle_kernel(float* __restrict__ 
   __shared__ float bsm[kSmallCap];
   __shared__ double red[32];
   __shared__ float meanb;
+  __shared__ float qs[kSmallQ];
   int ns[8], off[8], L = 0;
   {
     int n = n0, o = 0;
@@ -788,101 +866,99 @@ __global__ void __launch_bounds__(1024) small_vcycle_kernel(float* __restrict__ 
     xs[t] = 0.f;
     s += v;
   }
-  s = block_sum<1024>(s, red);
+  s = block_sum<kSmallThreads>(s, red);
   if (threadIdx.x == 0) meanb = (float)(s / N0);
   __syncthreads();
   for (int t = threadIdx.x; t < N0; t += blockDim.x) bsm[t] -= meanb;
   __syncthreads();
-  const int cycles = L > 1 ? kSmallCycles : 2;
-  for (int cyc = 0; cyc < cycles; ++cyc) {
-    // down
-    for (int l = 0; l < L - 1; ++l) {
-      const int n = ns[l];
-      float* x = xs + off[l];
-      const float* b = bsm + off[l];
-      for (int sw = 0; sw < kNu; ++sw) {
-        small_rbgs(x, b, n, 0);
-        small_rbgs(x, b, n, 1);
+  // down
+  for (int l = 0; l < L - 1; ++l) {
+    const int n = ns[l];
+    float* x = xs + off[l];
+    const float* b = bsm + off[l];
+    small_rbgs(x, b, n, kNu, 0);
+    const int nc = ns[l + 1];
+    float* xcn = xs + off[l + 1];
+    float* bcn = bsm + off[l + 1];
+    for (int t = threadIdx.x; t < nc * nc * nc; t += blockDim.x) {
+      const int I = t % nc, J = (t / nc) % nc, K = t / (nc * nc);
+      float acc = 0.f;
+      for (int ch = 0; ch < 8; ++ch) {
+        const int i = 2 * I + (ch & 1), j = 2 * J + ((ch >> 1) & 1), k = 2 * K + (ch >> 2);
+        const int p = (k * n + j) * n + i;
+        const float xv = x[p];
+        float lx = 0.f;
+        if (i > 0) lx += x[p - 1] - xv;
+        if (i < n - 1) lx += x[p + 1] - xv;
+        if (j > 0) lx += x[p - n] - xv;
+        if (j < n - 1) lx += x[p + n] - xv;
+        if (k > 0) lx += x[p - n * n] - xv;
+        if (k < n - 1) lx += x[p + n * n] - xv;
+        acc += b[p] - lx;
       }
-      const int nc = ns[l + 1];
-      float* xcn = xs + off[l + 1];
-      float* bcn = bsm + off[l + 1];
-      for (int t = threadIdx.x; t < nc * nc * nc; t += blockDim.x) {
-        const int I = t % nc, J = (t / nc) % nc, K = t / (nc * nc);
-        float acc = 0.f;
-        for (int ch = 0; ch < 8; ++ch) {
-          const int i = 2 * I + (ch & 1), j = 2 * J + ((ch >> 1) & 1), k = 2 * K + (ch >> 2);
-          const int p = (k * n + j) * n + i;
-          const float xv = x[p];
-          float lx = 0.f;
-          if (i > 0) lx += x[p - 1] - xv;
-          if (i < n - 1) lx += x[p + 1] - xv;
-          if (j > 0) lx += x[p - n] - xv;
-          if (j < n - 1) lx += x[p + n] - xv;
-          if (k > 0) lx += x[p - n * n] - xv;
-          if (k < n - 1) lx += x[p + n * n] - xv;
-          acc += b[p] - lx;
-        }
-        bcn[t] = 0.5f * acc;
-        xcn[t] = 0.f;
-      }
-      __syncthreads();
+      bcn[t] = 0.5f * acc;
+      xcn[t] = 0.f;
     }
-    // coarsest
-    {
-      const int n = ns[L - 1];
-      float* x = xs + off[L - 1];
-      const float* b = bsm + off[L - 1];
-      // a coarsest level of at most 4^3 below a hierarchy needs only a rough
-      // solve; a larger one (no hierarchy, e.g. an odd grid) is the whole solve
-      const int sweeps = (n <= 4 && L > 1) ? 2 * n + 8 : 2 * n * n + 16;
-      for (int sw = 0; sw < sweeps; ++sw) {
-        small_rbgs(x, b, n, 0);
-        small_rbgs(x, b, n, 1);
-      }
+    __syncthreads();
+  }
+  // coarsest
+  {
+    const int n = ns[L - 1];
+    float* x = xs + off[L - 1];
+    float* b = bsm + off[L - 1];
+    // a coarsest level of at most 4^3 below a hierarchy needs only a rough solve
+    if (n <= 4 && L > 1) {
+      small_rbgs(x, b, n, 2 * n + 8, 0);
+    } else {
+      small_basis(qs, n);
+      small_direct(x, b, n, qs, false);
     }
-    // up
-    for (int l = L - 2; l >= 0; --l) {
-      const int n = ns[l], nc = ns[l + 1];
-      float* x = xs + off[l];
-      const float* b = bsm + off[l];
-      const float* xcn = xs + off[l + 1];
-      for (int t = threadIdx.x; t < n * n * n; t += blockDim.x) {
-        const int i = t % n, j = (t / n) % n, k = t / (n * n);
-        x[t] += prolong_at(xcn, nc, i, j, k);
-      }
-      __syncthreads();
-      for (int sw = 0; sw < kNu; ++sw) {
-        small_rbgs(x, b, n, 1);
-        small_rbgs(x, b, n, 0);
-      }
+  }
+  // up
+  for (int l = L - 2; l >= 0; --l) {
+    const int n = ns[l], nc = ns[l + 1];
+    float* x = xs + off[l];
+    const float* b = bsm + off[l];
+    const float* xcn = xs + off[l + 1];
+    for (int t = threadIdx.x; t < n * n * n; t += blockDim.x) {
+      const int i = t % n, j = (t / n) % n, k = t / (n * n);
+      x[t] += prolong_at(xcn, nc, i, j, k);
     }
+    __syncthreads();
+    small_rbgs(x, b, n, kNu, 1);
   }
   for (int t = threadIdx.x; t < N0; t += blockDim.x) xg[t] = xs[t];
 }
 
 // The same hierarchy for L' with Gauss-Seidel in 8 colours ((i, j, k) mod 2:
 // no two cells of a colour are neighbours in the 27-point stencil), in place.
-__device__ void small_gs8(float* x, const float* b, int n, int color) {
-  const int N = n * n * n;
-  for (int t = threadIdx.x; t < N; t += blockDim.x) {
-    const int i = t % n, j = (t / n) % n, k = t / (n * n);
-    if (((i & 1) | ((j & 1) << 1) | ((k & 1) << 2)) != color) continue;
-    float acc = 0.f, ws = 0.f;
-    for (int dz = -1; dz <= 1; ++dz)
-      for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-          const int nz = (dx != 0) + (dy != 0) + (dz != 0);
-          if (nz < 2) continue;
-          const int qi = q1_fold(i + dx, n), qj = q1_fold(j + dy, n), qk = q1_fold(k + dz, n);
-          if (qi == i && qj == j && qk == k) continue;
-          const float w = nz == 2 ? 2.f : 1.f;
-          acc += w * x[(qk * n + qj) * n + qi];
-          ws += w;
-        }
-    x[t] = ws > 0.f ? (acc - b[t]) / ws : 0.f;
+// A thread owns one 2 x 2 x 2 block of cells (found once, not per colour) and
+// updates the block's cell of the pass's colour.
+__device__ void small_gs8(float* x, const float* b, int n, int sweeps, int first, int step) {
+  const int hc = (n + 1) >> 1;
+  const int row = threadIdx.x / hc;
+  const int i2 = 2 * ((int)threadIdx.x - row * hc), j2 = 2 * (row % hc), k2 = 2 * (row / hc);
+  for (int q = 0; q < 8 * sweeps; ++q) {
+    const int color = first + step * (q & 7);
+    const int i = i2 + (color & 1), j = j2 + ((color >> 1) & 1), k = k2 + (color >> 2);
+    if (i < n && j < n && k < n) {
+      float acc = 0.f, ws = 0.f;
+      for (int dz = -1; dz <= 1; ++dz)
+        for (int dy = -1; dy <= 1; ++dy)
+          for (int dx = -1; dx <= 1; ++dx) {
+            const int nz = (dx != 0) + (dy != 0) + (dz != 0);
+            if (nz < 2) continue;
+            const int qi = q1_fold(i + dx, n), qj = q1_fold(j + dy, n), qk = q1_fold(k + dz, n);
+            if (qi == i && qj == j && qk == k) continue;
+            const float w = nz == 2 ? 2.f : 1.f;
+            acc += w * x[(qk * n + qj) * n + qi];
+            ws += w;
+          }
+      const int t = (k * n + j) * n + i;
+      x[t] = ws > 0.f ? (acc - b[t]) / ws : 0.f;
+    }
+    __syncthreads();
   }
-  __syncthreads();
 }
 
 __device__ float small_q1_residual(const float* x, const float* b, int n, int i, int j, int k) {
@@ -901,7 +977,7 @@ __device__ float small_q1_residual(const float* x, const float* b, int n, int i,
   return b[p] - lx;
 }
 
-__global__ void __launch_bounds__(1024) small_vcycle_q1_kernel(float* __restrict__ xg, const float* __restrict__ bg,
+__global__ void __launch_bounds__(kSmallThreads) small_vcycle_q1_kernel(float* __restrict__ xg, const float* __restrict__ bg,
                                                                const float* __restrict__ shift, int n0,
                                                                const int* __restrict__ gate) {
   if (*gate) return;
@@ -909,6 +985,7 @@ __global__ void __launch_bounds__(1024) small_vcycle_q1_kernel(float* __restrict
   __shared__ float bsm[kSmallCap];
   __shared__ double red[32];
   __shared__ float meanb;
+  __shared__ float qs[kSmallQ];
   int ns[8], off[8], L = 0;
   {
     int n = n0, o = 0;
@@ -930,53 +1007,51 @@ __global__ void __launch_bounds__(1024) small_vcycle_q1_kernel(float* __restrict
     xs[t] = 0.f;
     s += v;
   }
-  s = block_sum<1024>(s, red);
+  s = block_sum<kSmallThreads>(s, red);
   if (threadIdx.x == 0) meanb = (float)(s / N0);
   __syncthreads();
   for (int t = threadIdx.x; t < N0; t += blockDim.x) bsm[t] -= meanb;
   __syncthreads();
-  const int cycles = L > 1 ? kSmallCycles : 2;
-  for (int cyc = 0; cyc < cycles; ++cyc) {
-    for (int l = 0; l < L - 1; ++l) {
-      const int n = ns[l];
-      float* x = xs + off[l];
-      const float* b = bsm + off[l];
-      for (int sw = 0; sw < kNu; ++sw)
-        for (int c = 0; c < 8; ++c) small_gs8(x, b, n, c);
-      const int nc = ns[l + 1];
-      float* xcn = xs + off[l + 1];
-      float* bcn = bsm + off[l + 1];
-      for (int t = threadIdx.x; t < nc * nc * nc; t += blockDim.x) {
-        const int I = t % nc, J = (t / nc) % nc, K = t / (nc * nc);
-        float acc = 0.f;
-        for (int ch = 0; ch < 8; ++ch)
-          acc += small_q1_residual(x, b, n, 2 * I + (ch & 1), 2 * J + ((ch >> 1) & 1), 2 * K + (ch >> 2));
-        bcn[t] = 0.5f * acc;
-        xcn[t] = 0.f;
-      }
-      __syncthreads();
+  for (int l = 0; l < L - 1; ++l) {
+    const int n = ns[l];
+    float* x = xs + off[l];
+    const float* b = bsm + off[l];
+    small_gs8(x, b, n, kNu, 0, 1);
+    const int nc = ns[l + 1];
+    float* xcn = xs + off[l + 1];
+    float* bcn = bsm + off[l + 1];
+    for (int t = threadIdx.x; t < nc * nc * nc; t += blockDim.x) {
+      const int I = t % nc, J = (t / nc) % nc, K = t / (nc * nc);
+      float acc = 0.f;
+      for (int ch = 0; ch < 8; ++ch)
+        acc += small_q1_residual(x, b, n, 2 * I + (ch & 1), 2 * J + ((ch >> 1) & 1), 2 * K + (ch >> 2));
+      bcn[t] = 0.5f * acc;
+      xcn[t] = 0.f;
     }
-    {
-      const int n = ns[L - 1];
-      float* x = xs + off[L - 1];
-      const float* b = bsm + off[L - 1];
-      const int sweeps = (n <= 4 && L > 1) ? 2 * n + 8 : 2 * n * n + 16;
-      for (int sw = 0; sw < sweeps; ++sw)
-        for (int c = 0; c < 8; ++c) small_gs8(x, b, n, c);
+    __syncthreads();
+  }
+  {
+    const int n = ns[L - 1];
+    float* x = xs + off[L - 1];
+    float* b = bsm + off[L - 1];
+    if (n <= 4 && L > 1) {
+      small_gs8(x, b, n, 2 * n + 8, 0, 1);
+    } else {
+      small_basis(qs, n);
+      small_direct(x, b, n, qs, true);
     }
-    for (int l = L - 2; l >= 0; --l) {
-      const int n = ns[l], nc = ns[l + 1];
-      float* x = xs + off[l];
-      const float* b = bsm + off[l];
-      const float* xcn = xs + off[l + 1];
-      for (int t = threadIdx.x; t < n * n * n; t += blockDim.x) {
-        const int i = t % n, j = (t / n) % n, k = t / (n * n);
-        x[t] += prolong_at(xcn, nc, i, j, k);
-      }
-      __syncthreads();
-      for (int sw = 0; sw < kNu; ++sw)
-        for (int c = 7; c >= 0; --c) small_gs8(x, b, n, c);
+  }
+  for (int l = L - 2; l >= 0; --l) {
+    const int n = ns[l], nc = ns[l + 1];
+    float* x = xs + off[l];
+    const float* b = bsm + off[l];
+    const float* xcn = xs + off[l + 1];
+    for (int t = threadIdx.x; t < n * n * n; t += blockDim.x) {
+      const int i = t % n, j = (t / n) % n, k = t / (n * n);
+      x[t] += prolong_at(xcn, nc, i, j, k);
     }
+    __syncthreads();
+    small_gs8(x, b, n, kNu, 7, -1);
   }
   for (int t = threadIdx.x; t < N0; t += blockDim.x) xg[t] = xs[t];
 }
@@ -1042,7 +1117,7 @@ int vcycle(wgeo_handle* h, int l, float* x0, const float* b0, const float* shift
   const float* b = (l == 0) ? b0 : h->levels[l].b;
   const float* shift = (l == 0) ? shift0 : nullptr;
   if (n <= kSmallN || l == h->nlevels - 1) {
-    small_vcycle_kernel<<<1, 1024, 0, s>>>(x, b, shift, n, gate);
+    small_vcycle_kernel<<<1, kSmallThreads, 0, s>>>(x, b, shift, n, gate);
     WGEO_LAUNCH_CHECK();
     return WGEO_OK;
   }
@@ -1799,7 +1874,7 @@ int vcycle_q1(wgeo_handle* h, int l, float* x0, const float* b0, const float* sh
   const float* b = (l == 0) ? b0 : h->levels[l].b;
   const float* shift = (l == 0) ? shift0 : nullptr;
   if (n <= kSmallN || l == h->nlevels - 1) {
-    small_vcycle_q1_kernel<<<1, 1024, 0, s>>>(x, b, shift, n, gate);
+    small_vcycle_q1_kernel<<<1, kSmallThreads, 0, s>>>(x, b, shift, n, gate);
     WGEO_LAUNCH_CHECK();
     return WGEO_OK;
   }
