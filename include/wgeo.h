@@ -98,7 +98,8 @@ typedef struct {
   int32_t spectral;          /* 1 (default): when res is a power of two from 32 to 512, MIXED mode
                                 takes each refinement step's correction from a direct spectral
                                 solve (the operator is diagonal in the cosine basis of the mirrored
-                                walls; always two steps), and FP32 mode solves once, directly;
+                                walls; always two steps), and FP32 mode solves once, directly; on
+                                every other res the adjoint solve does so, in two steps as well;
                                 0: multigrid V-cycles on every grid */
   int32_t reserved[3];
   double  tol_rel_adjoint;   /* adjoint solve: stop when ||g - A lambda|| <= tol * ||g|| (default 1e-7) */

@@ -17,6 +17,9 @@
 //   one-block kernel reduces the sums in a fixed order and tests
 //   ||r - mean r|| <= tol ||b - mean b||.  The correction solves
 //   L e = r - mean(r) with FP32 V-cycles.
+//   A direct spectral solve gives the correction instead where it is built:
+//   forward and adjoint on power-of-two grids (FFT passes, below), the adjoint
+//   on every other grid (dense transforms, spectral_dense.cu).
 // Plain FP32 (comparator): no refinement.  On power-of-two grids (with the
 //   spectral option) one direct FP32 spectral solve of L x = b - mean(b);
 //   elsewhere FP32 V-cycles directly on x32.  The residual and its norms are
@@ -1181,8 +1184,13 @@ constexpr int kDctTile = 32;      // lines per block: 16 warps, two lines each
 constexpr int kDctThreads = 512;
 constexpr unsigned kFull = 0xffffffffu;
 
-bool use_spectral(const wgeo_handle* h, int n) {
-  return h->opt.spectral && n >= 32 && n <= 512 && (n & (n - 1)) == 0;
+// Whether the FFT passes take this grid, and whether a solve's correction is a
+// direct spectral one: on the other grids the dense transforms
+// (spectral_dense.cu) give it to the adjoint solve, while forward solves keep
+// their V-cycles (and with them chi, warm starts and the plain FP32 mode).
+bool fft_grid(int n) { return n >= 32 && n <= 512 && (n & (n - 1)) == 0; }
+bool use_spectral(const wgeo_handle* h, int n, int mode) {
+  return h->opt.spectral && (fft_grid(n) || mode == 1);
 }
 
 __host__ __device__ constexpr int dct_ls(int n) { return (n + n / 32) | 1; }   // odd row stride
@@ -1829,7 +1837,7 @@ int spectral_solve(wgeo_handle* h, int n, float* e, const float* r, const int* g
     case 128: return spectral_passes<4>(h, e, r, gate, s);
     case 256: return spectral_passes<8>(h, e, r, gate, s);
     case 512: return spectral_passes<16>(h, e, r, gate, s);
-    default: return WGEO_ERR_INVALID_ARG;
+    default: return dense_solve(h, n, e, r, gate, s);
   }
 }
 
@@ -1845,6 +1853,7 @@ cudaError_t dct_attr() {
 // The twiddle and eigenvalue tables for n, and the shared-memory opt-in of the
 // pass kernels on the handle's device (host calls, kept out of any capture).
 int spectral_setup(wgeo_handle* h, int n, cudaStream_t s) {
+  if (!fft_grid(n)) return dense_setup(h, n, s);
   if (!h->dct_attr) {
     WGEO_CUDA_TRY(dct_attr<1>());
     WGEO_CUDA_TRY(dct_attr<2>());
@@ -1926,7 +1935,7 @@ int enqueue_part(wgeo_handle* h, int res, int mode, int part, int step, cudaGrap
     if (part == 1) {
       // plain FP32: on spectral grids one direct FP32 solve of L x = b - mean(b)
       // (no refinement), else one FP32 V-cycle on x in place
-      int rc = use_spectral(h, res) ? spectral_solve(h, res, h->chi32, h->b32, gate, s)
+      int rc = use_spectral(h, res, mode) ? spectral_solve(h, res, h->chi32, h->b32, gate, s)
                                     : vcycle(h, 0, h->chi32, h->b32, &ss->bmean32, false, gate, s);
       if (rc) return rc;
     }
@@ -1943,7 +1952,7 @@ int enqueue_part(wgeo_handle* h, int res, int mode, int part, int step, cudaGrap
   float* x32 = mode == 0 ? h->chi32 : h->lam32;
   if (part == 1) {
     // correction: V-cycles on L e = r - mean(r)
-    if (use_spectral(h, res)) {
+    if (use_spectral(h, res, mode)) {
       int rc = spectral_solve(h, res, h->e32, h->r32, gate, s);
       if (rc) return rc;
     } else {
@@ -2115,7 +2124,7 @@ int launch_solve_body(wgeo_handle* h, int res, int mode, bool cold, cudaStream_t
 // flag stays set until its test).  The iterations and their results are those
 // of the solve with the head.
 bool skip_head(const wgeo_handle* h, int res, int mode, bool cold) {
-  return cold && use_spectral(h, res) && !h->opt.galerkin && (mode == 1 || h->opt.precision == WGEO_PREC_MIXED);
+  return cold && use_spectral(h, res, mode) && !h->opt.galerkin && (mode == 1 || h->opt.precision == WGEO_PREC_MIXED);
 }
 
 // Enqueues one solve.  The launch sequence depends only on (res, mode,
@@ -2125,7 +2134,7 @@ bool skip_head(const wgeo_handle* h, int res, int mode, bool cold) {
 int launch_solve(wgeo_handle* h, int res, int mode, bool cold, cudaStream_t s) {
   const int64_t N = (int64_t)res * res * res;
   SolveState* ss = mode == 0 ? &h->dstate->fwd : &h->dstate->bwd;
-  if (use_spectral(h, res)) {
+  if (use_spectral(h, res, mode)) {
     int rc = spectral_setup(h, res, s);
     if (rc) return rc;
   }
@@ -2172,7 +2181,7 @@ int launch_solve_body(wgeo_handle* h, int res, int mode, bool cold, cudaStream_t
   // first is exact to FP32 rounding): always take both, so that chi, and the
   // adjoint's right-hand side built from it, carry no solver error
   // (plain FP32 takes its one direct solve)
-  const int min_steps = use_spectral(h, res) ? (fp32_plain ? 1 : 2) : 0;
+  const int min_steps = use_spectral(h, res, mode) ? (fp32_plain ? 1 : 2) : 0;
   const bool skip = skip_head(h, res, mode, cold);
   if (skip && mode == 0)
     WGEO_CUDA_TRY(cudaMemcpyAsync(h->r32, h->b32, sizeof(float) * (size_t)res * res * res, cudaMemcpyDeviceToDevice, s));

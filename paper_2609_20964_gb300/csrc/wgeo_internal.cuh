@@ -400,6 +400,10 @@ struct wgeo_handle {
   float* dct_skl = nullptr;      //   the same at k = a + R brev5(j)
   int dct_n = 0;                 // n the tables hold (0: none yet)
   bool dct_attr = false;         // shared-memory opt-in of the pass kernels done (per device)
+  // dense cosine transforms of the other grids: forward basis, inverse basis, eigenvalue factors
+  float* dense_tab = nullptr;
+  int dense_n = 0;               // n the tables hold (0: none yet)
+  bool dense_attr = false;
 
   // points
   int* pcell = nullptr;          // packed central cell per point (original order); -1 = skipped
@@ -532,6 +536,10 @@ int launch_bin_sort_splat(wgeo_handle* h, const float* points, const float* norm
 int launch_unpack_bins(wgeo_handle* h, int* out, cudaStream_t s);
 // solver.cu
 int launch_solve(wgeo_handle* h, int res, int mode, bool cold, cudaStream_t s);
+// spectral_dense.cu: the direct correction on grids without an FFT pass
+size_t dense_table_floats(int max_res);
+int dense_setup(wgeo_handle* h, int n, cudaStream_t s);
+int dense_solve(wgeo_handle* h, int n, float* e, const float* r, const int* gate, cudaStream_t s);
 // surface.cu
 int launch_isovalue(wgeo_handle* h, const float* points, int64_t n, int res, cudaStream_t s);
 int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_out, cudaStream_t s);
