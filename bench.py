@@ -419,7 +419,7 @@ def fp32_peak():
 FP32_PEAK_TFLOPS = None   # set by fp32_peak() once a device is current
 FP32_PEAK_KIND = None
 FLOPS_PER_TRI_TEST = 40.0      # FP32 operations of one point-triangle distance
-STAGE_KERNEL = {"sdf": ("sdf_kernel", "paper_2609_20964_gb300/csrc/surface.cu")}
+STAGE_KERNEL = {"sdf": ("sdf_patch_kernel", "paper_2609_20964_gb300/csrc/surface.cu")}
 
 
 def source_digest(rel_paths):

@@ -134,8 +134,9 @@ typedef struct {
   int64_t  n_triangles;      /* triangles extracted by the last forward */
   int64_t  n_points_used;    /* finite points used by the last forward */
   double   h;                /* cell size of the last forward */
-  int64_t  sdf_node_visits;  /* with stage_timing = 2: octree nodes entered by the distance search (per warp) */
-  int64_t  sdf_leaf_visits;  /* ... leaves entered (per warp) */
+  int64_t  sdf_node_visits;  /* with stage_timing = 2: octree nodes entered by the distance search (per
+                                block of nodes, or per node where it searches one by one) */
+  int64_t  sdf_leaf_visits;  /* ... leaves entered (the same) */
   int64_t  sdf_tri_tests;    /* ... point-triangle distance evaluations (per node, i.e. per lane) */
   double   backward_dc;      /* dL/dc of the last backward */
   int64_t  sdf_tie_nodes;    /* with stage_timing = 2: nodes whose nearest triangle was a float32

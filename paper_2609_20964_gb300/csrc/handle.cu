@@ -20,7 +20,7 @@ constexpr size_t kAlign = 256;
 struct Layout {
   size_t total = 0;
   size_t off_b32, off_chi32, off_chi64, off_r32, off_e32, off_phi, off_ctri, off_dphi, off_dchi64,
-      off_lam64, off_lam32, off_levels, off_dct, off_dense, off_pcell, off_pfrac, off_pnrm, off_srec, off_tile_count,
+      off_lam64, off_lam32, off_levels, off_dct, off_dense, off_axis, off_pcell, off_pfrac, off_pnrm, off_srec, off_tile_count,
       off_tile_off, off_tile_cursor, off_brick_count, off_brick_off, off_leaf_off, off_leaf_cnt, off_tris, off_tris_lo, off_tris_s, off_cell_pyr, off_pyr, off_pyr_sums, off_pyr_rth, off_partials,
       off_scan, off_state, off_dp_cell, off_dp_count, off_dp_off, off_dp_cursor, off_dp_scan, off_dp_tmp,
       off_dp_sorted, off_dp_key, off_dp_gbox, off_or_scal;
@@ -60,6 +60,7 @@ Layout make_layout(int R, int64_t P, const wgeo_options& opt) {
   L.off_levels = take(c, 4 * lev);
   L.off_dct = take(c, 8 * (512 + 160 + 512 + 16 + 512 + 520) + 4 * (512 + 512));   // spectral tables, n <= 512
   L.off_dense = take(c, opt.spectral ? sizeof(float) * dense_table_floats(R) : 0);
+  L.off_axis = take(c, 4 * 3 * (size_t)R);
   const size_t Pp = (size_t)(P > 0 ? P : 1);
   L.off_pcell = take(c, 4 * Pp);
   L.off_pfrac = take(c, 16 * Pp);
@@ -290,6 +291,7 @@ int wgeo_create(wgeo_handle** out, int32_t max_res, int64_t max_points, const wg
   h->dct_tw = reinterpret_cast<float2*>(h->dct_skl + 512);
   h->dct_wq = h->dct_tw + 512;
   h->dense_tab = (float*)(a + L.off_dense);
+  h->axis = (float*)(a + L.off_axis);
   h->pcell = (int*)(a + L.off_pcell);
   h->pfrac = (float4*)(a + L.off_pfrac);
   h->pnrm = keep ? (float4*)(a + L.off_pnrm) : nullptr;

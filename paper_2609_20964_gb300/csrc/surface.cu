@@ -27,6 +27,7 @@
 // chi >= c, -1 where chi < c (the marching-cubes surface separates the two node
 // classes, so this is the parity of crossings of any ray from the node).
 #include <math.h>
+#include <stddef.h>
 
 #include <algorithm>
 
@@ -379,8 +380,15 @@ __global__ void mc_count_kernel(const unsigned* __restrict__ bits, SurfParams g,
   }
 }
 
+// The triangle total and its status, and the node coordinates per axis (the
+// distance search reads them instead of forming them in FP64 at every node).
 __global__ void mc_total_kernel(const int* __restrict__ brick_off, int nbricks, int64_t cap,
-                                int* __restrict__ leaf_off, DevState* st) {
+                                int* __restrict__ leaf_off, DevState* st, SurfParams g, float* __restrict__ axis) {
+  for (int t = threadIdx.x; t < 3 * g.res; t += blockDim.x) {
+    const int a = t / g.res, i = t - a * g.res;
+    axis[t] = (float)(g.lo[a] + (i + 0.5) * g.h);
+  }
+  if (threadIdx.x != 0) return;
   const long long T = brick_off[nbricks];
   st->ntris = T;
   leaf_off[8 * (int64_t)nbricks] = brick_off[nbricks];
@@ -615,19 +623,17 @@ __device__ __forceinline__ int leaf_index(int lx, int ly, int lz, int nb) {
   return 8 * br + ((lx & 1) | ((ly & 1) << 1) | ((lz & 1) << 2));
 }
 
-constexpr float kPuckPad = 1e-5f;   // relative inflation: rounding of the bound stays conservative
-
-// 10-bit hash of a marching-cubes vertex (its global edge id).
-__device__ __forceinline__ unsigned vertex_hash10(float gid_bits) {
-  return (__float_as_uint(gid_bits) * 0x9E3779B1u) >> 22;
-}
+// Inflation of a puck's radius and half-thickness, for the float rounding of
+// the offsets they are the largest of (relative) and of the ~48-bit vertices
+// behind the float32 ones (of the coordinates' magnitude).  What the distance
+// of a query rounds is left to puck_dist2.
+constexpr float kPuckRel = 2e-6f;
+constexpr float kPuckAbs = 2e-7f;
 
 // Search record of a triangle for the distance search: vertex a and the edge
-// vectors ab, ac with the Gram entries |ab|^2 and |ac|^2 (ab.ac is formed
-// where it is used), the reciprocals the Voronoi regions divide by (0 for a
-// zero-length edge or a collapsed triangle), and in the slot of ab.ac the
-// 10-bit hashes of the three vertices (bits 0-9 a, 10-19 b, 20-29 c), which
-// name a closest vertex or edge without another memory access.
+// vectors ab, ac with the Gram entries |ab|^2, ab.ac and |ac|^2, and the
+// reciprocals the Voronoi regions divide by (0 for a zero-length edge or a
+// collapsed triangle).
 // With the vertices' low parts (lo, may be null) the edge vectors are the
 // float32 roundings of the differences of the ~48-bit vertices, not the
 // differences of the float32 vertices: their directions then carry float32
@@ -646,8 +652,7 @@ __device__ __forceinline__ void write_search_record(const Tri& tr, const Tri* lo
   const float3 cr = cross3(ab, ac);
   const float det = dot3(cr, cr);   // = |ab|^2 |ac|^2 - (ab.ac)^2, without the cancellation
   rec[0] = make_float4(a.x, a.y, a.z, e00);
-  const unsigned vk = vertex_hash10(tr.a.w) | (vertex_hash10(tr.b.w) << 10) | (vertex_hash10(tr.c.w) << 20);
-  rec[1] = make_float4(ab.x, ab.y, ab.z, __uint_as_float(vk));
+  rec[1] = make_float4(ab.x, ab.y, ab.z, dot3(ab, ac));
   rec[2] = make_float4(ac.x, ac.y, ac.z, e11);
   rec[3] = make_float4(e00 > 0.f ? 1.f / e00 : 0.f, e11 > 0.f ? 1.f / e11 : 0.f, ebc > 0.f ? 1.f / ebc : 0.f,
                        det > 0.f ? 1.f / det : 0.f);
@@ -719,9 +724,23 @@ __device__ __forceinline__ void fit_puck(const Tri* __restrict__ tris, int64_t q
       r = fmaxf(r, sqrtf(rho2));
     }
   }
-  const float pad = kPuckPad * (fabsf(cc.x) + fabsf(cc.y) + fabsf(cc.z) + r + th) + 1e-7f;
-  A = make_float4(cc.x, cc.y, cc.z, r * (1.f + kPuckPad) + pad);
-  B = make_float4(nv.x, nv.y, nv.z, th * (1.f + kPuckPad) + pad);
+  const float pad = kPuckRel * (r + th) + kPuckAbs * (fabsf(cc.x) + fabsf(cc.y) + fabsf(cc.z));
+  A = make_float4(cc.x, cc.y, cc.z, r + pad);
+  B = make_float4(nv.x, nv.y, nv.z, th + pad);
+}
+
+// Rank of the q-th triangle of a leaf in a depth-first walk of the octree that
+// takes children from the last to the first (the leaf's Morton code, 9 bits an
+// axis, descending): the order in which the search ranks equal distances.
+__device__ __forceinline__ unsigned walk_rank(int lx, int ly, int lz, int q) {
+  auto spread = [](unsigned v) {   // nine bits, two zeros between each
+    v = (v | (v << 16)) & 0x030000ffu;
+    v = (v | (v << 8)) & 0x0300f00fu;
+    v = (v | (v << 4)) & 0x030c30c3u;
+    return (v | (v << 2)) & 0x09249249u;
+  };
+  const unsigned m = spread((unsigned)lx) | (spread((unsigned)ly) << 1) | (spread((unsigned)lz) << 2);
+  return ((0x07ffffffu - m) << 5) | (unsigned)min(q, 31);
 }
 
 // Leaf pucks, pass 2 (live leaves): the triangles' search records, the
@@ -729,7 +748,7 @@ __device__ __forceinline__ void fit_puck(const Tri* __restrict__ tris, int64_t q
 // cube of the leaf that holds triangles, stored at the slot of the cube's
 // first triangle (cell_pyr[2 q0], [2 q0 + 1]); leaf_cnt packs the cubes'
 // triangle counts, 4 bits per cube in the leaf's cube order.
-__global__ void puck_leaf_kernel(const Tri* __restrict__ tris, const Tri* __restrict__ tris_lo,
+__global__ void puck_leaf_kernel(const Tri* __restrict__ tris, Tri* __restrict__ tris_lo,
                                  const int* __restrict__ leaf_off, const unsigned* __restrict__ leaf_cnt, int nb,
                                  int64_t cap, const int* __restrict__ live, const DevState* __restrict__ st,
                                  float4* __restrict__ pyr, float4* __restrict__ tris_s,
@@ -748,6 +767,7 @@ __global__ void puck_leaf_kernel(const Tri* __restrict__ tris, const Tri* __rest
       if (tris_lo) {
         const Tri tl = tris_lo[q];
         write_search_record(tr, &tl, tris_s + kTriRec * q);
+        tris_lo[q].a.w = __uint_as_float(walk_rank(lx, ly, lz, (int)(q - s0)));
       } else {
         write_search_record(tr, nullptr, tris_s + kTriRec * q);
       }
@@ -775,17 +795,20 @@ __global__ void puck_leaf_kernel(const Tri* __restrict__ tris, const Tri* __rest
 // Tight puck of an internal node at level l >= 1 (dim d_l; level 1 = bricks):
 // axis and centre from its own triangles, radius and half-thickness from
 // their vertices (two passes over the bricks it covers).
-// Squared distance from p to the solid cylinder of a puck (INF when empty).
+// Squared distance from p to the solid cylinder of a puck (INF when empty),
+// from below: every term that p's distance d to the centre rounds (z and the
+// hardware reciprocal square root, a few 1e-7 d; the difference d^2 - z^2, a
+// few 1e-7 d^2) is taken low by 1e-6 of it.  (An inflation of the pucks by 1e-5
+// of the coordinates covered the same: 0.008 cells of thickness at 512^3,
+// which at 150 cells from the surface admits 1.5 cells more on every side.)
 __device__ __forceinline__ float puck_dist2(const float3 p, const float4 A, const float4 B) {
   if (A.w < 0.f) return INFINITY;
   const float3 d = make_float3(p.x - A.x, p.y - A.y, p.z - A.z);
   const float z = d.x * B.x + d.y * B.y + d.z * B.z;
-  // rho from the hardware reciprocal square root (a few ulp), scaled down by
-  // 1e-6 so that it stays below the exact value: a lower bound still
-  const float x2 = fmaxf(d.x * d.x + d.y * d.y + d.z * d.z - z * z, 0.f);
-  const float rho = x2 * rsqrtf(fmaxf(x2, 1e-30f)) * (1.f - 1e-6f);
-  const float dz = fmaxf(fabsf(z) - B.w, 0.f);
-  const float dr = fmaxf(rho - A.w, 0.f);
+  const float x2 = fmaxf(fmaf(d.x * d.x + d.y * d.y + d.z * d.z, 1.f - 1e-6f, -z * z), 0.f);
+  const float rho = x2 * rsqrtf(fmaxf(x2, 1e-30f));
+  const float dz = fmaxf(fmaf(fabsf(z), 1.f - 1e-6f, -B.w), 0.f);
+  const float dr = fmaxf(fmaf(rho, 1.f - 1e-6f, -A.w), 0.f);
   return dz * dz + dr * dr;
 }
 
@@ -917,9 +940,9 @@ __global__ void puck_finalize_kernel(float4* __restrict__ pyr, const float4* __r
     float3 c, ax;
     node_frame(s0, s1, c, ax);
     const float r = __uint_as_float(rth[2 * a]), th = __uint_as_float(rth[2 * a + 1]);
-    const float pad = kPuckPad * (fabsf(c.x) + fabsf(c.y) + fabsf(c.z) + r + th) + 1e-7f;
-    pyr[2 * gi] = make_float4(c.x, c.y, c.z, r * (1.f + kPuckPad) + pad);
-    pyr[2 * gi + 1] = make_float4(ax.x, ax.y, ax.z, th * (1.f + kPuckPad) + pad);
+    const float pad = kPuckRel * (r + th) + kPuckAbs * (fabsf(c.x) + fabsf(c.y) + fabsf(c.z));
+    pyr[2 * gi] = make_float4(c.x, c.y, c.z, r + pad);
+    pyr[2 * gi + 1] = make_float4(ax.x, ax.y, ax.z, th + pad);
   }
 }
 
@@ -956,7 +979,7 @@ __global__ void puck_mask_kernel(float4* __restrict__ pyr, PyrInfo pi) {
 namespace {
 
 constexpr int kWarps = 4;          // warps per CTA
-constexpr int kStack = 96;         // per-warp traversal stack
+constexpr int kStack = 96;         // per-warp traversal stack (exact queries)
 
 // Float32 rounding of one point-triangle distance, as a bound used to detect
 // near-ties: relative to the distance, plus an absolute part for the rounding
@@ -964,7 +987,6 @@ constexpr int kStack = 96;         // per-warp traversal stack
 constexpr float kTieRel = 4e-7f;
 constexpr float kTieAbs = 1.5e-7f;
 constexpr int kCand = 4;           // smallest float32 distances kept per node
-constexpr int kSdfCoarse = 2;      // stride of the coarsest (unseeded) search pass
 
 struct TieSlots {
   int2* p[2];   // the two float-float iterate buffers; the one not current is free
@@ -978,14 +1000,12 @@ struct TieSlots {
 // p - y = ap - v ab - w ac is formed relative to a, so its rounding scales
 // with the distance and the edge length rather than with the coordinates.
 
-__device__ __forceinline__ float tri_dist2_rec(const float3 p, const float4* __restrict__ rec, float& v, float& w,
-                                               unsigned& vk) {
+__device__ __forceinline__ float tri_dist2_rec(const float3 p, const float4* __restrict__ rec, float& v, float& w) {
   const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
   const float3 ap = make_float3(p.x - r0.x, p.y - r0.y, p.z - r0.z);
   const float d1 = r1.x * ap.x + r1.y * ap.y + r1.z * ap.z;   // ab . ap
   const float d2 = r2.x * ap.x + r2.y * ap.y + r2.z * ap.z;   // ac . ap
   rec_weights(ap, d1, d2, r0, r1, r2, r3, v, w);
-  vk = __float_as_uint(r1.w);
   const float rx = ap.x - v * r1.x - w * r2.x;
   const float ry = ap.y - v * r1.y - w * r2.y;
   const float rz = ap.z - v * r1.z - w * r2.z;
@@ -993,19 +1013,36 @@ __device__ __forceinline__ float tri_dist2_rec(const float3 p, const float4* __r
 }
 __device__ __forceinline__ float tri_dist2_rec(const float3 p, const float4* __restrict__ rec) {
   float v, w;
-  unsigned vk;
-  return tri_dist2_rec(p, rec, v, w, vk);
+  return tri_dist2_rec(p, rec, v, w);
 }
 
-// Key (32-bit hash; callers keep its top bits) of a node's closest feature on triangle t, from the weights
-// (v, w) of its closest point y = a + v ab + w ac and the record's vertex
-// hashes: a vertex (weights 0 / 1) by its hash, an edge (one weight 0, or
-// v = 1 - w) by its two, a face by the triangle.  Triangles that share the
-// closest vertex or edge give the same key.
-__device__ __forceinline__ unsigned feature_key(float v, float w, unsigned vk, int t) {
-  const unsigned ha = vk & 1023u, hb = (vk >> 10) & 1023u, hc = (vk >> 20) & 1023u;
-  unsigned x;
+// Key (32-bit hash) of a node's closest feature on triangle t, from the weights
+// (v, w) of its closest point y = a + v ab + w ac and the edge ids of the
+// triangle's vertices: a vertex (weights 0 / 1) by its id, an edge (one weight
+// 0, or v = 1 - w) by its two, a face by the triangle.  Triangles that share
+// the closest vertex or edge give the same key; vertices never collide, other
+// pairs with probability 2^-32.
+__device__ __forceinline__ unsigned feature_key(float v, float w, const Tri* __restrict__ tri, int t) {
+  auto mix = [](unsigned x) {
+    x *= 0x9E3779B1u;
+    return x ^ (x >> 15);
+  };
+  const bool onb = v == 1.f && w == 0.f, onc = w == 1.f && v == 0.f, ona = v == 0.f && w == 0.f;
+  const bool face = !(w == 0.f || v == 0.f || v == 1.f - w);
+  if (face) return mix(mix((unsigned)t) + 0x7F4A7C15u);
+  const unsigned ga = mix(__float_as_uint(tri[t].a.w)), gb = mix(__float_as_uint(tri[t].b.w)),
+                 gc = mix(__float_as_uint(tri[t].c.w));
+  if (ona || onb || onc) return ona ? ga : onb ? gb : gc;
+  const unsigned p = w == 0.f ? ga : v == 0.f ? ga : gb, q = w == 0.f ? gb : gc;
+  return mix((min(p, q) * 0x85EBCA6Bu) ^ max(p, q));
+}
+
+// Class of the same feature: a hash of ten bits per vertex (sdf_tie_kernel).
+__device__ __forceinline__ unsigned feature_class(float v, float w, const Tri* __restrict__ tri, int t) {
+  auto hash10 = [](float gid) { return (__float_as_uint(gid) * 0x9E3779B1u) >> 22; };
   auto edge = [](unsigned p, unsigned q) { return (1u << 20) | (min(p, q) << 10) | max(p, q); };
+  const unsigned ha = hash10(tri[t].a.w), hb = hash10(tri[t].b.w), hc = hash10(tri[t].c.w);
+  unsigned x;
   if (w == 0.f) {
     x = (v == 0.f) ? ha : (v == 1.f ? hb : edge(ha, hb));
   } else if (v == 0.f) {
@@ -1018,37 +1055,14 @@ __device__ __forceinline__ unsigned feature_key(float v, float w, unsigned vk, i
   return ((x * 0x9E3779B1u) ^ 0x7F4A7C15u) * 0x85EBCA6Bu;
 }
 
-// The same distance in float-float for the near-tie decisions.  Only ap and
-// the residual need the extra precision: a region chosen wrongly near a
-// region boundary, and rounding of the weights (v, w), change |p - y| only to
-// second order (the residual is normal to the directions they move y in), so
-// the region and the weights come from the float32 path; ap is formed in
-// float-float from the float-float node position, v ab + w ac from exact
-// products, and |p - y|^2 in float-float.
-__device__ __forceinline__ Ff two_prod_ff(float a, float b) {
-  const float p = __fmul_rn(a, b);
-  return Ff(p, __fmaf_rn(a, b, -p));
-}
-
-__device__ __forceinline__ Ff tri_dist2_rec_ff(const Vec3<Ff> p, const float4* __restrict__ rec) {
-  const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
-  const Ff apx = p.x - Ff(r0.x), apy = p.y - Ff(r0.y), apz = p.z - Ff(r0.z);
-  const float3 ap = make_float3(apx.hi, apy.hi, apz.hi);
-  const float d1 = r1.x * ap.x + r1.y * ap.y + r1.z * ap.z;
-  const float d2 = r2.x * ap.x + r2.y * ap.y + r2.z * ap.z;
-  float v, w;
-  rec_weights(ap, d1, d2, r0, r1, r2, r3, v, w);
-  const Ff rx = apx - (two_prod_ff(v, r1.x) + two_prod_ff(w, r2.x));
-  const Ff ry = apy - (two_prod_ff(v, r1.y) + two_prod_ff(w, r2.y));
-  const Ff rz = apz - (two_prod_ff(v, r1.z) + two_prod_ff(w, r2.z));
-  return rx * rx + ry * ry + rz * rz;
-}
-
-// The same on the ~48-bit vertices (float32 vertex + its low part, see
-// mc_emit_kernel): a, ab and ac in float-float, so the distance is that of
-// the refined surface to ~1e-14 relative and two candidates are ranked as
-// the exact (FP64) mesh ranks them unless they tie to that level.  The region
-// and the weights still come from the float32 record (second-order effect).
+// The same distance in float-float for the near-tie decisions, on the ~48-bit
+// vertices (float32 vertex + its low part, see mc_emit_kernel): a, ab, ac and
+// ap in float-float, so the distance is that of the refined surface to ~1e-14
+// relative and two candidates are ranked as the exact (FP64) mesh ranks them
+// unless they tie to that level.  The Voronoi region and the weights (v, w)
+// come from the float32 record: a region chosen wrongly near a region boundary,
+// and rounding of the weights, change |p - y| only to second order (the
+// residual is normal to the directions they move y in).
 __device__ __forceinline__ Ff tri_dist2_ff_exact(const Vec3<Ff> p, const float4* __restrict__ rec, const Tri& hi,
                                                  const Tri& lo) {
   const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
@@ -1079,322 +1093,948 @@ __device__ __forceinline__ unsigned pack_node(int lev, int x, int y, int z) {
   return ((unsigned)lev << 27) | ((unsigned)z << 18) | ((unsigned)y << 9) | (unsigned)x;
 }
 
-// Warp-cooperative exact distance search: a warp owns a 4 x 4 x 2 patch of
-// nodes and walks the octree once for all of them (a subtree is entered when
-// its bound beats the current cut of at least one lane); in a leaf, the
-// triangles of each MC cube whose own puck beats some lane's cut are tested
-// by every lane against its own node with the same (broadcast) triangle.
+// ---- Exact distance search over the grid nodes.
 //
 // Exactness at near-ties: two triangles whose distances differ by less than
 // the float32 rounding may be ranked either way, and the closest point (and
-// with it the vertex gradient of Eqs. 35-36) differs between them.  Each lane
-// keeps its kCand smallest float32 distances (four: triangles sharing the
-// closest edge tie exactly, so candidates come in pairs) and prunes against
-// the best plus a rounding margin; when the second lies within that margin
-// the node is a near-tie: it is appended to tie_list, the ids of the
-// candidates within the margin go to tie_a, tie_b and tie_cd at the same list
-// position (-1 for none), and sdf_tie_kernel re-decides it in float-float.  Without TIES (no closest
-// triangle is kept) the search keeps the float32 minimum alone, which is
-// within the same rounding of the exact distance.
+// with it the vertex gradient of Eqs. 35-36) differs between them.  Each node
+// keeps its kCand smallest float32 distances, one per closest feature, and
+// prunes against the best plus a rounding margin; when the second lies within
+// that margin the node is a near-tie: it is appended to tie_list, the ids of
+// the candidates within the margin go to tie_a, tie_b and tie_cd at the same
+// list position (-1 for none), and sdf_tie_kernel re-decides it in
+// float-float.  Without TIES (no closest triangle is kept) the search keeps
+// the float32 minimum alone, which is within the same rounding of the exact
+// distance.
 //
-// Coarse to fine passes over nested lattices: pass `stride` S handles the
-// nodes whose coordinates are all multiples of S but not all multiples of 2S
-// (the coarsest pass, S = kSdfCoarse, takes all its lattice's nodes and
-// starts from nothing).  A finer pass starts from the closest triangles of
-// the up to 8 nodes of the 2S lattice around its node (seed_ids, written by
-// every pass for its nodes): real triangle distances, so the cut is an upper
-// bound from the start and the search mostly has to certify.
-template <bool COUNT, bool TIES>
-__global__ void __launch_bounds__(kWarps * 32, 10) sdf_kernel(const float* __restrict__ chi, SurfParams g,
-                                                          DevState* __restrict__ st,
-                                                          const float4* __restrict__ tris_s, int id_bits,
-                                                          const int* __restrict__ leaf_off, int64_t cap,
-                                                          const float4* __restrict__ pyr, PyrInfo pi,
-                                                          float* __restrict__ phi, float* __restrict__ sdf_out,
-                                                          int* __restrict__ ctri, int* __restrict__ tie_a,
-                                                          int* __restrict__ tie_b, TieSlots tie_cd,
-                                                          int* __restrict__ tie_list,
-                                                          int* __restrict__ seed_ids, int stride,
-                                                          const unsigned* __restrict__ leaf_cnt,
-                                                          const float4* __restrict__ cell_pyr) {
-  __shared__ uint2 s_node[kWarps][kStack];   // (packed level and coordinates, pyramid index)
-  __shared__ int s_off[12];
-  __shared__ int s_dim[12];
-  if (threadIdx.x < 12) {
-    s_off[threadIdx.x] = pi.off[threadIdx.x];
-    s_dim[threadIdx.x] = pi.dim[threadIdx.x];
-  }
-  __syncthreads();
-  const int n = g.res;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // CTA covers 8 x 8 x 2 nodes of this pass's lattice: warp w -> (4 (w & 1),
-  // 4 (w >> 1)) in x, y
-  const int S = stride;
-  const bool seeded = S < kSdfCoarse;
-  const int nl = (n + S - 1) / S;
-  const int ntx = (nl + 7) / 8, nty = (nl + 7) / 8;
-  const int bx = blockIdx.x % ntx, by = (blockIdx.x / ntx) % nty, bz = blockIdx.x / (ntx * nty);
-  const int i = S * (bx * 8 + 4 * (w & 1) + (lane & 3));
-  const int j = S * (by * 8 + 4 * (w >> 1) + ((lane >> 2) & 3));
-  const int k = S * (bz * 2 + (lane >> 4));
-  const bool valid = (i < n) && (j < n) && (k < n) && (!seeded || ((i | j | k) & S));
-  const int ic = min(i, n - 1), jc = min(j, n - 1), kc = min(k, n - 1);
-  const float3 p = make_float3((float)(g.lo[0] + (ic + 0.5) * g.h), (float)(g.lo[1] + (jc + 0.5) * g.h),
-                               (float)(g.lo[2] + (kc + 0.5) * g.h));
-  constexpr int NC = TIES ? kCand : 1;
-  float coord = 0.f;
+// Nested lattices, coarse to fine: sdf_node_kernel searches the nodes of the
+// coarsest lattice, a warp per node; sdf_patch_kernel then takes the lattices
+// of half the stride in turn, a block per 8 x 8 x 4 nodes, seeded with the
+// closest triangles of the coarser lattice's nodes around them; blocks with too
+// many candidates (around a point far from everything, like a sphere's centre,
+// every triangle is one) leave their nodes on a list that sdf_node_kernel
+// takes at the end.
+//
+// Bound: instruction issue (72% of the slots; a node's answer is 60 flops, the
+// proof that no other triangle is nearer the rest).  Per warp of 32 nodes at
+// 128^3 (star body, 76,000 triangles) the finest pass runs 12,000 instructions
+// against 25,000 of a warp that walks the octree for its 32 nodes by itself,
+// testing each popped puck and each triangle for all of them: 0.7 for the
+// seeds, 2 for the block's walk, 1 + 2.5 for the patch's cubes (of 240 in the
+// block's reach, 74 in the patch's and 6.7 in a node's), 3 for 19 triangle
+// tests a node and 2 for its 3 exact ones.  Search stage before -> now, ms:
+// 0.79 -> 0.32 (64^3, 16,384 points), 2.79 -> 1.61 (128^3), 16.4 -> 11.9
+// (256^3), 137 -> 90 (512^3); 1.47 -> 0.30 on a 64^3 sphere, whose centre kept
+// one warp busy for all of it.
+
+// What the search reads and writes (device pointers of the handle).
+struct Search {
+  const float4* tris_s;
+  const Tri* tris;
+  const Tri* tris_lo;       // a.w: walk_rank
+  const int* leaf_off;
+  const unsigned* leaf_cnt;
+  const float4* pyr;
+  const float4* cell_pyr;
+  const float* axis;        // node coordinates, [3][res]
+  const float* chi;
+  DevState* st;
+  int64_t cap;
+  int n;                    // nodes per axis
+  int nb;                   // bricks per axis
+  float h;
+  float coord;              // largest |coordinate| of the box
+  float* phi;
+  float* sdf_out;
+  int* ctri;
+  int* tie_a;
+  int* tie_b;
+  TieSlots tie_cd;
+  int* tie_list;
+  int* seed_ids;            // closest triangle of every node of the lattices done so far
+  int* defer;               // nodes left to sdf_node_kernel
+};
+
+// The candidate list of one node: the NC smallest distances, one entry per
+// closest feature (by feature_key; with TIES alone), in registers.  Triangles
+// sharing the closest vertex (often six of them) or edge tie exactly and would
+// otherwise fill the list and push out a distinct surface point at the same
+// distance (a node on the medial axis), which the tie pass must see.  Entries
+// are ordered by distance, equal ones with the node's seeds first (s: its eight
+// of them, may be null) and then by walk_rank, so the list does not depend on
+// the order in which triangles come; each comes once.
+__device__ __forceinline__ bool comes_first(int t, int u, const Tri* __restrict__ tris_lo, const int* s) {
+  if (s) {
+    int st = 8, su = 8;
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-    coord = fmaxf(coord, (float)fmax(fabs(g.lo[a]), fabs(g.lo[a] + n * g.h)));
-  const float mabs = kTieAbs * coord;
+    for (int q = 7; q >= 0; --q) {
+      if (s[q] == t) st = q;
+      if (s[q] == u) su = q;
+    }
+    if (st != su) return st < su;
+  }
+  const unsigned rt = __float_as_uint(tris_lo[t].a.w), ru = __float_as_uint(tris_lo[u].a.w);
+  return rt < ru || (rt == ru && t < u);
+}
+
+template <bool TIES>
+struct Cands {
+  static constexpr int NC = TIES ? kCand : 1;
   float cd[NC];
   int ct[NC];
+  unsigned ck[NC];
+  float cut;        // a near-tie's squared distance is at most this
+  __device__ __forceinline__ void init(bool valid) {
 #pragma unroll
-  for (int q = 0; q < NC; ++q) {
-    cd[q] = INFINITY;
-    ct[q] = -1;
+    for (int q = 0; q < NC; ++q) {
+      cd[q] = INFINITY;
+      ct[q] = -1;
+      ck[q] = 0u;
+    }
+    cut = valid ? INFINITY : -INFINITY;
   }
-  float cut = valid ? INFINITY : -INFINITY;   // a lane without a node never asks for a subtree
-  // With id_bits > 0 (near-tie handles; triangle ids below 2^id_bits - 1,
-  // id_bits <= 24) each list entry carries the top 32 - id_bits bits of its
-  // closest feature's key (feature_key) above the id, and the list holds one
-  // entry per closest feature:
-  // triangles sharing the closest vertex (often six of them) or edge tie
-  // exactly and would otherwise fill the list and push out a distinct surface
-  // point at the same distance (a node on the medial axis), which the tie
-  // pass must see.  Entries merge when their keys match; both lie within the
-  // rounding margin of the best, so a key collision can at most leave a tie
-  // to the float32 ranking.
-  const bool keyed = TIES && id_bits > 0;
-  const int idmask = keyed ? (int)((1u << id_bits) - 1u) : -1;
-  auto margin2 = [&](float x) {
-    const float r = sqrtf(x) * (1.f + kTieRel) + mabs;
+  // the exact test of triangle t against p, and its place in the list
+  __device__ __forceinline__ void offer(const float3 p, int t, const Search& S, const int* seeds) {
+    float v, w;
+    const float d2 = tri_dist2_rec(p, S.tris_s + kTriRec * (int64_t)t, v, w);
+    if (!TIES) {
+      if (d2 < cd[0] || (d2 == cd[0] && t < ct[0])) {
+        cd[0] = d2;
+        ct[0] = t;
+      }
+      return;
+    }
+    if (!(d2 <= cd[NC - 1])) return;
+    const unsigned key = feature_key(v, w, S.tris, t);
+    bool before[NC];   // whether t comes before entry q (false, ..., true, ...)
+    int at = NC - 1;   // the entry it replaces: its feature's, else the last
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      before[q] = d2 < cd[q];
+      if (d2 == cd[q] && ct[q] != -1) before[q] = comes_first(t, ct[q], S.tris_lo, seeds);
+      if (ct[q] != -1 && ck[q] == key) at = q;
+    }
+#pragma unroll
+    for (int q = NC - 1; q >= 0; --q) {
+      if (q > at || !before[q]) continue;
+      const bool down = q > 0 && before[q > 0 ? q - 1 : 0];   // the entry above moves here
+      cd[q] = down ? cd[q > 0 ? q - 1 : 0] : d2;
+      ct[q] = down ? ct[q > 0 ? q - 1 : 0] : t;
+      ck[q] = down ? ck[q > 0 ? q - 1 : 0] : key;
+    }
+  }
+  __device__ __forceinline__ void swap(int a, int b) {
+    const float tf = cd[a];
+    cd[a] = cd[b];
+    cd[b] = tf;
+    const int ti = ct[a];
+    ct[a] = ct[b];
+    ct[b] = ti;
+    const unsigned tk = ck[a];
+    ck[a] = ck[b];
+    ck[b] = tk;
+  }
+  // the cut that goes with the best distance
+  __device__ __forceinline__ float reach(float mabs) const {
+    if (!TIES) return cd[0];
+    const float r = sqrtf(cd[0]) * (1.f + kTieRel) + mabs;
     return r * r;
-  };
-  // candidate list insertion (sorted, duplicates of a listed triangle ignored)
-  auto offer = [&](float d2, int t, float v, float w, unsigned vk) {
-    if (!(d2 < cut && d2 < cd[NC - 1])) return;
-    int e = t;
-    int at = NC - 1;
-    if (keyed) {
-      const unsigned key = feature_key(v, w, vk, t) >> id_bits;
-      e = t | (int)(key << id_bits);
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        if ((ct[q] & idmask) == t) return;
-        if (ct[q] != -1 && ((unsigned)ct[q] >> id_bits) == key) {
-          if (!(d2 < cd[q])) return;      // the listed entry of this feature stays
-          at = q;                         // replaced in place, then moved up
-        }
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < NC; ++q)
-        if (ct[q] == t) return;
-    }
-#pragma unroll
-    for (int q = 0; q < NC; ++q) {   // static indices: the list stays in registers
-      if (q == at) {
-        cd[q] = d2;
-        ct[q] = e;
-      }
-    }
-#pragma unroll
-    for (int q = NC - 1; q > 0; --q) {
-      if (q <= at && cd[q] < cd[q - 1]) {
-        const float tf = cd[q];
-        cd[q] = cd[q - 1];
-        cd[q - 1] = tf;
-        const int ti = ct[q];
-        ct[q] = ct[q - 1];
-        ct[q - 1] = ti;
-      }
-    }
-    if (TIES) {
-      cut = margin2(cd[0]);
-    } else {
-      cut = cd[0];
-    }
-  };
-  if (seeded && valid) {
-    // seeds: the closest triangles of the 2S-lattice nodes around this node
-    const int S2 = 2 * S;
-    const int i0 = i & ~(S2 - 1), j0 = j & ~(S2 - 1), k0 = k & ~(S2 - 1);
-#pragma unroll 1
-    for (int q = 0; q < 8; ++q) {
-      const int ii = i0 + S2 * (q & 1), jj = j0 + S2 * ((q >> 1) & 1), kk = k0 + S2 * (q >> 2);
-      if (ii >= n || jj >= n || kk >= n) continue;
-      const int t = seed_ids[lin3(ii, jj, kk, n)];
-      if (t >= 0) {
-        float v, w;
-        unsigned vk;
-        const float d2 = tri_dist2_rec(p, tris_s + kTriRec * (int64_t)t, v, w, vk);
-        offer(d2, t, v, w, vk);
-      }
-    }
   }
-  uint2* stk = s_node[w];
-  int sp = 0;
-  const int top = pi.nlev - 1;
-  const int nb = (s_dim[0] + 1) / 2;
-  if (lane == 0) stk[0] = make_uint2(pack_node(top, 0, 0, 0), (unsigned)s_off[top]);
-  sp = 1;
-  unsigned long long c_nodes = 0, c_leaves = 0, c_tests = 0;
-  // the warp's nodes' bounding box: centre and half-diagonal, widened so that
-  // float rounding keeps the box bound below every lane's exact bound
-  float bc[3], br;
-  {
-    const float pv[3] = {p.x, p.y, p.z};
-    float r2 = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      float lo = pv[a], hi = pv[a];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      }
-      bc[a] = 0.5f * (lo + hi);
-      const float e = 0.5f * (hi - lo);
-      r2 += e * e;
-    }
-    br = sqrtf(r2) * (1.f + 1e-5f) + 1e-7f * coord;
-  }
-  const float3 pb = make_float3(bc[0], bc[1], bc[2]);
-  __syncwarp();
-  while (sp > 0) {
-    --sp;
-    const uint2 en = stk[sp];
-    __syncwarp();
-    const unsigned e = en.x;
-    const int gi = (int)en.y;
-    const int lev = (int)(e >> 27);
-    const int x = (int)(e & 511u), y = (int)((e >> 9) & 511u), z = (int)((e >> 18) & 511u);
-    const float4 An = pyr[2 * gi];
-    const float lb = puck_dist2(p, An, pyr[2 * gi + 1]);
-    if (!__any_sync(0xffffffffu, lb < cut)) continue;
-    if (COUNT) ++c_nodes;
-    if (lev == 0) {
-      const int li = leaf_index(x, y, z, nb);
-      const int s1 = (int)min((int64_t)leaf_off[li + 1], cap);
-      if (COUNT) ++c_leaves;
-      // the leaf's cubes in order; a cube's triangles are tested when its
-      // own puck beats the cut of at least one lane
-      unsigned cn = leaf_cnt[li];
-      int q0 = leaf_off[li];
-#pragma unroll 1
-      for (; cn != 0u; cn >>= 4) {
-        const int q1 = min(q0 + (int)(cn & 15u), s1);
-        if (q0 < q1 &&
-            __any_sync(0xffffffffu, puck_dist2(p, cell_pyr[2 * q0], cell_pyr[2 * q0 + 1]) < cut)) {
-          if (COUNT) c_tests += 32ull * (unsigned long long)(q1 - q0);
-          for (int t = q0; t < q1; ++t) {
-            float v, w;
-            unsigned vk;
-            const float d2 = tri_dist2_rec(p, tris_s + kTriRec * t, v, w, vk);
-            offer(d2, t, v, w, vk);
-          }
-        }
-        q0 += (int)(cn & 15u);
-      }
-      continue;
-    }
-    const int dc = s_dim[lev - 1];
-    const int cbase = s_off[lev - 1];
-    // children, one per lane (lanes 0-7): kept when their bound from the
-    // warp's box (the puck's distance to the box centre less the box's
-    // half-diagonal, a lower bound for every node in it) beats the largest
-    // lane cut; pushed far-to-near by that bound in the unseeded pass, in
-    // child order in the seeded ones (their cuts start near their final
-    // values, so the order saves little and the ranking costs 8 shuffles).
-    // Each lane's own bound is checked when a child is popped, so a child is
-    // bounded per lane once.
-    const unsigned cmask = __float_as_uint(An.w) & 0xffu;
-    const float maxcut = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(cut, 0.f))));
-    bool keep = false;
-    float key = INFINITY;
-    uint2 ent = make_uint2(0u, 0u);
-    if (lane < 8 && ((cmask >> lane) & 1u)) {
-      const int cx = 2 * x + (lane & 1), cy = 2 * y + ((lane >> 1) & 1), cz = 2 * z + (lane >> 2);
-      const int cg = cbase + (cz * dc + cy) * dc + cx;
-      const float dcen = sqrtf(puck_dist2(pb, pyr[2 * cg], pyr[2 * cg + 1])) * (1.f - 2e-6f) - br;
-      key = dcen > 0.f ? dcen * dcen : 0.f;
-      keep = key < maxcut;
-      ent = make_uint2(pack_node(lev - 1, cx, cy, cz), (unsigned)cg);
-    }
-    const unsigned kept = __ballot_sync(0xffffffffu, keep);
-    const int nc = __popc(kept);
-    int rank = 0;   // kept children nearer than this one (ties by lane)
-    if (seeded) {
-      rank = nc - 1 - __popc(kept & ((1u << lane) - 1u));
-    } else {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float kq = __shfl_sync(0xffffffffu, key, q);
-        if (((kept >> q) & 1u) && (kq < key || (kq == key && q < lane))) ++rank;
-      }
-    }
-    const int slot = sp + nc - 1 - rank;
-    if (keep && slot < kStack) stk[slot] = ent;
-    sp = min(sp + nc, kStack);
-    __syncwarp();
-  }
-  const bool tie = TIES && valid && ct[NC > 1 ? 1 : 0] != -1 && cd[NC > 1 ? 1 : 0] <= cut;
-  if (COUNT) {
-    const unsigned long long nt = (unsigned long long)__popc(__ballot_sync(0xffffffffu, tie));
-    if (lane == 0) {
-      atomicAdd(&st->sdf_cnt[0], c_nodes);
-      atomicAdd(&st->sdf_cnt[1], c_leaves);
-      atomicAdd(&st->sdf_cnt[2], c_tests);
-      atomicAdd(&st->sdf_cnt[3], nt);
-    }
-  }
-  const int64_t o = lin3(i, j, k, n);
+};
+
+// Results of the warp's nodes (lane with `valid`: linear node o): distance and
+// sign, closest triangle, and the near-tie list (one atomic per warp; the
+// candidates at the same list position, so that the tie pass reads them
+// coalesced).
+template <bool COUNT, bool TIES>
+__device__ __forceinline__ void store_nodes(const Search& S, const Cands<TIES>& c, bool valid, int64_t o, bool seed,
+                                            int lane) {
+  constexpr int NC = Cands<TIES>::NC;
+  const bool tie = TIES && valid && c.ct[NC > 1 ? 1 : 0] != -1 && c.cd[NC > 1 ? 1 : 0] <= c.cut;
   int tie_at = 0;
   if (TIES) {
-    // near-tie nodes go to a compact list (one atomic per warp), so that the
-    // tie pass runs full warps over them alone; their candidates are stored
-    // at the same list position (read coalesced by the tie pass)
     const unsigned m = __ballot_sync(0xffffffffu, tie);
     if (m) {
       const int leader = __ffs(m) - 1;
       unsigned base = 0;
-      if (lane == leader) base = atomicAdd(&st->ntie, (unsigned)__popc(m));
+      if (lane == leader) {
+        base = atomicAdd(&S.st->ntie, (unsigned)__popc(m));
+        if (COUNT) atomicAdd(&S.st->sdf_cnt[3], (unsigned long long)__popc(m));
+      }
       base = __shfl_sync(0xffffffffu, base, leader);
       tie_at = (int)(base + __popc(m & ((1u << lane) - 1u)));
-      if (tie) tie_list[tie_at] = (int)o;
+      if (tie) S.tie_list[tie_at] = (int)o;
     }
   }
   if (!valid) return;
-  const float val = sqrtf(cd[0]);
-  const int bt = ct[0] == -1 ? -1 : (ct[0] & idmask);
-  const float sgn = (chi[o] >= st->c_up) ? 1.f : -1.f;
-  phi[o] = sgn * val;
-  if (sdf_out) sdf_out[o] = sgn * val;
-  if (ctri) ctri[o] = bt;
-  if (S > 1) seed_ids[o] = bt;
+  const int bt = c.ct[0];
+  const float val = (S.chi[o] >= S.st->c_up ? 1.f : -1.f) * sqrtf(c.cd[0]);
+  S.phi[o] = val;
+  if (S.sdf_out) S.sdf_out[o] = val;
+  if (S.ctri) S.ctri[o] = bt;
+  if (seed) S.seed_ids[o] = bt;
   if (TIES && tie) {
-    tie_a[tie_at] = bt;
-    tie_b[tie_at] = ct[NC > 1 ? 1 : 0] & idmask;
-    const int c2 = ct[NC > 2 ? 2 : 0], c3 = ct[NC > 3 ? 3 : 0];
-    tie_cd.p[st->fwd.xidx ^ 1][tie_at] = make_int2(cd[NC > 2 ? 2 : 0] <= cut && c2 != -1 ? (c2 & idmask) : -1,
-                                                   cd[NC > 3 ? 3 : 0] <= cut && c3 != -1 ? (c3 & idmask) : -1);
+    S.tie_a[tie_at] = bt;
+    S.tie_b[tie_at] = c.ct[NC > 1 ? 1 : 0];
+    int more[2] = {-1, -1};
+#pragma unroll
+    for (int q = 2; q < NC; ++q)
+      if (c.cd[q] <= c.cut && c.ct[q] != -1) more[q - 2] = c.ct[q];
+    S.tie_cd.p[S.st->fwd.xidx ^ 1][tie_at] = make_int2(more[0], more[1]);
   }
 }
 
-// Float-float decision between the float32 near-tie candidates of a node:
-// distances (tri_dist2_ff_exact on the ~48-bit vertices when their low parts
-// exist, else tri_dist2_rec_ff on the float32 ones) from the node position
-// rounded once from double, the smaller wins; equal distances (a shared edge or vertex: the
-// same closest point) take the smaller triangle index.  The node coordinates come from per-axis
-// float-float tables built once per block, and chi >= c (c double) is tested
-// as chi >= the smallest float not below c, so no node needs FP64.
+// Octree entries waiting on a warp's stack: pack_node's word and the node's
+// child-occupancy mask, known when the node was bounded, so a pop needs no
+// memory.  Up to four nodes are popped at a time, their 32 children bounded one
+// per lane.  Four are taken only while the stack holds kPopFour entries or
+// fewer, then one by one: a pop of one node of level l leaves at most 7 more
+// entries per level below it, so the stack stays below kPopFour - 4 + 32 + 7 *
+// 9 (at most 10 levels).
+constexpr int kPopFour = 60;
+constexpr int kSrchStack = 160;
+static_assert(kPopFour - 4 + 32 + 7 * 9 <= kSrchStack, "search stack");
 
-__global__ void sdf_tie_kernel(const float* __restrict__ chi, SurfParams g, const DevState* __restrict__ st,
-                               const float4* __restrict__ tris_s, const Tri* __restrict__ tris,
-                               const Tri* __restrict__ tris_lo, const int* __restrict__ tie_a,
-                               const int* __restrict__ tie_b, TieSlots tie_cd, const int* __restrict__ tie_list,
-                               float* __restrict__ phi, float* __restrict__ sdf_out, int* __restrict__ ctri) {
+// One leaf's cube of a lane: its first triangle and triangle count, from the
+// leaf's triangle offset and its cubes' counts (4 bits each).
+__device__ __forceinline__ void leaf_cube(const Search& S, int li, int cube, int& q0, int& cnt) {
+  const unsigned cn = S.leaf_cnt[li];
+  const unsigned below = cn & ((1u << (4 * cube)) - 1u);
+  const unsigned pairs = (below & 0x0f0f0f0fu) + ((below >> 4) & 0x0f0f0f0fu);
+  q0 = S.leaf_off[li] + (int)((pairs * 0x01010101u) >> 24);
+  cnt = (int)((cn >> (4 * cube)) & 15u);
+  if ((int64_t)q0 + cnt > S.cap) cnt = max((int)(S.cap - q0), 0);
+}
+
+// Whether some point of a box may have its closest surface point, or a near-tie
+// with it, in a puck.  With y a surface point, p0 the box's centre and e its
+// half extents, any point p of the box is at most |p - y| from the surface,
+// and for a point c of the puck |p - c|^2 - |p - y|^2 is linear in p: its
+// least value over the box is |p0 - c|^2 - |p0 - y|^2 - 2 sum_a e_a |c - y|_a.
+// So the puck is out when its distance to p0 exceeds |p0 - y| by more than
+// that sum's bound over the puck's bounding sphere.  Unlike a bound from the
+// distance to the box alone, whose slack grows with the distance to the
+// surface, this one depends on the lateral offset c - y only.  Each of the
+// box's reference points y (the closest points of its corner nodes) has to
+// admit the puck: over a flat surface one of them alone admits offsets of
+// twice the box's extent on the far side, and the opposite corners' together
+// leave just the box's own footprint.
+// refs: y and |p0 - y|^2 widened by reach_of; N of them, at the indices of
+// ref_at (all eight corners, or four that share no edge).
+__device__ __forceinline__ constexpr int ref_at(int n, int q) { return n == 8 ? q : q == 0 ? 0 : q == 1 ? 3 : q == 2 ? 5 : 6; }
+template <int N>
+__device__ __forceinline__ bool puck_reaches(const float3 p0, const float4* refs, const float3 e, float elen,
+                                             const float4 A, const float4 B) {
+  const float d = puck_dist2(p0, A, B) * (1.f - 1e-6f) - 2.00002f * elen * (A.w + B.w);
+  bool in = true;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const float4 y = refs[ref_at(N, q)];
+    const float s = e.x * fabsf(A.x - y.x) + e.y * fabsf(A.y - y.y) + e.z * fabsf(A.z - y.z);
+    in = in && d <= fmaf(2.00002f, s, y.w);
+  }
+  return in;
+}
+
+// |p0 - y|^2 widened by the margin of a near-tie at the box's farthest point
+// from y (kTieRel, kTieAbs) and by the float rounding of y, p0 and the
+// squares.
+__device__ __forceinline__ float reach_of(const float3 p0, const float3 y, float elen, float coord) {
+  const float3 d = sub3(p0, y);
+  const float u = dot3(d, d);
+  const float m = sqrtf(u) + elen;
+  return u + 2.f * m * (1e-6f * m + 5e-7f * coord);
+}
+
+// Squared distance from p to a triangle without branches, to rank triangles:
+// the least of the three clamped edges and, when the projection falls inside,
+// the face, each as a quadratic form about vertex a (stationary in the
+// weights, so their rounding enters to second order).  Its error is below 1e-6
+// (|p - a|^2), a cancellation that tri_dist2_rec avoids; |p - a|^2 exceeds the
+// squared distance by at most the squared longest edge (3 h^2) where the
+// closest point lies on the triangle.
+__device__ __forceinline__ float tri_dist2_fast(const float3 p, const float4* __restrict__ rec) {
+  const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
+  const float3 ap = make_float3(p.x - r0.x, p.y - r0.y, p.z - r0.z);
+  const float s = ap.x * ap.x + ap.y * ap.y + ap.z * ap.z;
+  const float d1 = r1.x * ap.x + r1.y * ap.y + r1.z * ap.z;
+  const float d2 = r2.x * ap.x + r2.y * ap.y + r2.z * ap.z;
+  const float e00 = r0.w, e01 = r1.w, e11 = r2.w;
+  const float m1 = -2.f * d1, m2 = -2.f * d2;
+  const float t1 = __saturatef(d1 * r3.x), t2 = __saturatef(d2 * r3.y);
+  const float q1 = fmaf(t1, fmaf(t1, e00, m1), s), q2 = fmaf(t2, fmaf(t2, e11, m2), s);
+  const float g = e00 - e01, db = (d2 - d1) + g;            // bc . bp
+  const float t3 = __saturatef(db * r3.z);
+  const float q3 = fmaf(t3, fmaf(t3, g + (e11 - e01), -2.f * db), (s + m1) + e00);
+  const float v = (e11 * d1 - e01 * d2) * r3.w, w = (e00 * d2 - e01 * d1) * r3.w;
+  const float qf = fmaf(v, fmaf(v, e00, fmaf(2.f * w, e01, m1)), fmaf(w, fmaf(w, e11, m2), s));
+  const bool in = fminf(fminf(v, w), 1.f - (v + w)) >= 0.f;
+  const float q = fminf(fminf(q1, q2), q3);
+  return fmaxf(in ? fminf(q, qf) : q, 0.f);
+}
+
+// The cut that goes with a distance of tri_dist2_fast: margin2 widened by its
+// error (the square root by the hardware's approximation, from above).
+__device__ __forceinline__ float fast_cut(float q, float mabs, float h2) {
+  const float m = 2.f * mabs;
+  return fmaf(q, 1.f + 4e-6f, fmaf(2.001f * m, q * rsqrtf(fmaxf(q, 1e-30f)), fmaf(m, m, 1e-5f * h2)));
+}
+
+// Closest point to p on triangle t (its search record).
+__device__ __forceinline__ float3 closest_on(const float3 p, const float4* __restrict__ rec) {
+  const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
+  const float3 ap = make_float3(p.x - r0.x, p.y - r0.y, p.z - r0.z);
+  float v, w;
+  rec_weights(ap, r1.x * ap.x + r1.y * ap.y + r1.z * ap.z, r2.x * ap.x + r2.y * ap.y + r2.z * ap.z, r0, r1, r2, r3, v,
+              w);
+  return make_float3(r0.x + (v * r1.x + w * r2.x), r0.y + (v * r1.y + w * r2.y), r0.z + (v * r1.z + w * r2.z));
+}
+
+// ---- a warp per node: the coarsest lattice (LIST false: every stride-th node
+// from nothing, after a descent to the nearest leaf) or the deferred nodes
+// (LIST true: from the closest triangle found so far).  The 32 lanes bound 32
+// octree children, then 32 cubes, then test 32 triangles at a time against the
+// one node by tri_dist2_fast; the cut is the warp's smallest, and the triangles
+// within it wait for the exact test.
+constexpr int kNodeTris = 192;   // triangles waiting: below 32, plus 32 cubes of at most 5
+template <bool COUNT, bool TIES, bool LIST>
+__global__ void __launch_bounds__(kWarps * 32) sdf_node_kernel(const __grid_constant__ Search S,
+                                                               const __grid_constant__ PyrInfo pi, int stride) {
+  __shared__ unsigned s_stk[kWarps][kSrchStack];
+  __shared__ unsigned char s_msk[kWarps][kSrchStack];
+  __shared__ int s_leaf[kWarps][40];
+  __shared__ int s_tri[kWarps][kNodeTris];
+  __shared__ int s_hit[kWarps][64];
+  __shared__ float s_hq[kWarps][64];
+  __shared__ int s_off[12], s_dim[12];
+  if (threadIdx.x < 12) {
+    s_off[threadIdx.x] = (int)pi.off[threadIdx.x];
+    s_dim[threadIdx.x] = pi.dim[threadIdx.x];
+  }
+  __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  unsigned* stk = s_stk[w];
+  unsigned char* msk = s_msk[w];
+  int* leaf = s_leaf[w];
+  int* tri = s_tri[w];
+  int* hit = s_hit[w];
+  float* hq = s_hq[w];
+  const int n = S.n;
+  const int nl = (n + stride - 1) / stride;
+  const unsigned total = LIST ? S.st->ndefer : (unsigned)nl * nl * nl;
+  const int top = pi.nlev - 1;
+  const unsigned root_mask = __float_as_uint(S.pyr[2 * (int64_t)s_off[top]].w) & 0xffu;
+  const bool empty = S.pyr[2 * (int64_t)s_off[top]].w < 0.f;
+  const float mabs = TIES ? kTieAbs * S.coord : 0.f, h2 = S.h * S.h;
+  for (unsigned it = blockIdx.x * kWarps + w; it < total; it += gridDim.x * kWarps) {
+    int i, j, k;
+    if (LIST) {
+      const unsigned o = (unsigned)S.defer[it];
+      const unsigned row = o / (unsigned)n;
+      i = (int)(o - row * n), j = (int)(row % n), k = (int)(row / n);
+    } else {
+      const unsigned row = it / (unsigned)nl;
+      i = stride * (int)(it - row * nl), j = stride * (int)(row % nl), k = stride * (int)(row / nl);
+    }
+    const int64_t o = lin3(i, j, k, n);
+    const float3 p = make_float3(S.axis[i], S.axis[n + j], S.axis[2 * n + k]);
+    Cands<TIES> c;
+    c.init(true);
+    unsigned long long c_nodes = 0, c_leaves = 0, c_tests = 0;
+    float cut = INFINITY;   // of the fast distances
+    int nhit = 0;
+    // the waiting triangles still within the cut, moved together
+    auto drop_hits = [&]() {
+      int kept = 0;
+#pragma unroll
+      for (int q = 0; q < 64; q += 32) {
+        const int t = hit[q + lane];
+        const float d = hq[q + lane];
+        const bool in = q + lane < nhit && d < cut;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (in) {
+          hit[kept + __popc(m & below)] = t;
+          hq[kept + __popc(m & below)] = d;
+        }
+        kept += __popc(m);
+        __syncwarp();
+      }
+      nhit = kept;
+    };
+    // ... into the lanes' candidate lists
+    auto run_hits = [&]() {
+      for (int q = lane; q < nhit; q += 32) c.offer(p, hit[q], S, nullptr);
+      nhit = 0;
+      __syncwarp();
+    };
+    auto test = [&](bool on, int t) {
+      if (COUNT) c_tests += (unsigned)__popc(__ballot_sync(0xffffffffu, on));
+      float q = INFINITY;
+      if (on) q = tri_dist2_fast(p, S.tris_s + kTriRec * (int64_t)t);
+      const bool in = q < cut;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (m) {
+        cut = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(in ? fminf(cut, fast_cut(q, mabs, h2)) : cut)));
+        if (in) {
+          hit[nhit + __popc(m & below)] = t;
+          hq[nhit + __popc(m & below)] = q;
+        }
+        nhit += __popc(m);
+        __syncwarp();
+        if (nhit > 32) {
+          drop_hits();
+          if (nhit > 32) run_hits();
+        }
+      }
+    };
+    if (LIST) {
+      // its cube finds the seed again: only the cut is kept
+      const int seed = S.seed_ids[o];
+      test(lane == 0 && seed >= 0, seed);
+      nhit = 0;
+    } else if (!empty) {
+      // descent by the children's bounds; the leaf's triangles give the first cut
+      int x = 0, y = 0, z = 0;
+      unsigned mask = root_mask;
+      for (int lev = top; lev > 0; --lev) {
+        const int dc = s_dim[lev - 1];
+        float key = INFINITY;
+        unsigned cm = 0;
+        if (lane < 8 && ((mask >> lane) & 1u)) {
+          const int cx = 2 * x + (lane & 1), cy = 2 * y + ((lane >> 1) & 1), cz = 2 * z + (lane >> 2);
+          const int64_t cg = s_off[lev - 1] + ((int64_t)cz * dc + cy) * dc + cx;
+          const float4 A = S.pyr[2 * cg];
+          key = puck_dist2(p, A, S.pyr[2 * cg + 1]);
+          cm = __float_as_uint(A.w) & 0xffu;
+        }
+        const unsigned kb = __float_as_uint(key);
+        const int at = __ffs(__ballot_sync(0xffffffffu, kb == __reduce_min_sync(0xffffffffu, kb))) - 1;
+        mask = __shfl_sync(0xffffffffu, cm, at);
+        x = 2 * x + (at & 1), y = 2 * y + ((at >> 1) & 1), z = 2 * z + ((at >> 2) & 1);
+      }
+      const int li = leaf_index(x, y, z, S.nb);
+      const int q0 = S.leaf_off[li], q1 = (int)min((int64_t)S.leaf_off[li + 1], S.cap);
+      for (int q = q0; q < q1; q += 32) test(q + lane < q1, min(q + lane, q1 - 1));
+      nhit = 0;   // the leaf's cubes come again
+    }
+    int sp = 0, nlf = 0, nt = 0;
+    if (!empty) {
+      if (lane == 0) {
+        stk[0] = pack_node(top, 0, 0, 0);
+        msk[0] = (unsigned char)root_mask;
+      }
+      sp = 1;
+    }
+    __syncwarp();
+    while (sp > 0 || nlf > 0 || nt > 0) {
+      if (nt >= 32 || (sp == 0 && nlf == 0)) {
+        // 32 triangles
+        const int m = min(nt, 32);
+        nt -= m;
+        const int t = tri[nt + min(lane, m - 1)];
+        test(lane < m, t);
+        __syncwarp();
+      } else if (nlf >= 4 || sp == 0) {
+        // the cubes of four leaves
+        const int m = min(nlf, 4);
+        nlf -= m;
+        if (COUNT) c_leaves += m;
+        int q0 = 0, cnt = 0;
+        if ((lane >> 3) < m) leaf_cube(S, leaf[nlf + (lane >> 3)], lane & 7, q0, cnt);
+        if (cnt > 0 && !(puck_dist2(p, S.cell_pyr[2 * (int64_t)q0], S.cell_pyr[2 * (int64_t)q0 + 1]) < cut)) cnt = 0;
+        int at = cnt;   // inclusive prefix sum of the counts
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, at, d);
+          if (lane >= d) at += v;
+        }
+        const int all = __shfl_sync(0xffffffffu, at, 31);
+        at += nt - cnt;
+        for (int q = 0; q < cnt; ++q) tri[at + q] = q0 + q;
+        nt += all;
+        __syncwarp();
+      } else {
+        // the children of up to four nodes
+        const int m = sp <= kPopFour ? min(sp, 4) : 1;
+        sp -= m;
+        const int sl = lane >> 3, ch = lane & 7;
+        unsigned e = 0, mask = 0;
+        if (sl < m) {
+          e = stk[sp + sl];
+          mask = msk[sp + sl];
+        }
+        __syncwarp();
+        if (COUNT) c_nodes += m;
+        bool keep = false;
+        const int lev = (int)(e >> 27);
+        const int cx = 2 * (int)(e & 511u) + (ch & 1), cy = 2 * (int)((e >> 9) & 511u) + ((ch >> 1) & 1),
+                  cz = 2 * (int)((e >> 18) & 511u) + (ch >> 2);
+        unsigned cm = 0;
+        if ((mask >> ch) & 1u) {
+          const int dc = s_dim[lev - 1];
+          const int64_t cg = s_off[lev - 1] + ((int64_t)cz * dc + cy) * dc + cx;
+          const float4 A = S.pyr[2 * cg];
+          keep = puck_dist2(p, A, S.pyr[2 * cg + 1]) < cut;
+          cm = __float_as_uint(A.w) & 0xffu;
+        }
+        const bool lf = keep && lev == 1;
+        const unsigned mn = __ballot_sync(0xffffffffu, keep && !lf), ml = __ballot_sync(0xffffffffu, lf);
+        if (lf) {
+          leaf[nlf + __popc(ml & below)] = leaf_index(cx, cy, cz, S.nb);
+        } else if (keep) {
+          const int at = sp + __popc(mn & below);
+          stk[at] = pack_node(lev - 1, cx, cy, cz);
+          msk[at] = (unsigned char)cm;
+        }
+        sp += __popc(mn);
+        nlf += __popc(ml);
+        __syncwarp();
+      }
+    }
+    drop_hits();
+    Cands<TIES> r;
+    r.init(true);
+    constexpr int NC = Cands<TIES>::NC;
+    run_hits();
+    // the lanes' lists merged: the smallest entry of all, its feature (and its
+    // triangle) dropped everywhere, and again
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const unsigned kb = __float_as_uint(c.cd[0]);
+      const unsigned best = __reduce_min_sync(0xffffffffu, kb);
+      // equal distances: as in the list (without ranks by the triangle index)
+      const bool head = kb == best && c.ct[0] != -1;
+      const unsigned order = !head ? 0xffffffffu : TIES ? __float_as_uint(S.tris_lo[c.ct[0]].a.w) : (unsigned)c.ct[0];
+      const unsigned least = __reduce_min_sync(0xffffffffu, order);
+      const unsigned id = __reduce_min_sync(0xffffffffu, head && order == least ? (unsigned)c.ct[0] : 0xffffffffu);
+      const int own = __ffs(__ballot_sync(0xffffffffu, id != 0xffffffffu && c.ct[0] == (int)id)) - 1;
+      const unsigned key = __shfl_sync(0xffffffffu, c.ck[0], max(own, 0));
+      if (id != 0xffffffffu) {
+        r.cd[q] = __uint_as_float(best);
+        r.ct[q] = (int)id;
+      }
+#pragma unroll
+      for (int a = 0; a < NC; ++a) {
+        if (c.ct[a] != -1 && id != 0xffffffffu &&
+            (c.ct[a] == (int)id || (TIES && c.ck[a] == key))) {
+          c.cd[a] = INFINITY;
+          c.ct[a] = -1;
+        }
+      }
+      // the dropped entry (at most one: a lane lists a feature once) moves to the end
+#pragma unroll
+      for (int a = 0; a + 1 < NC; ++a)
+        if (c.cd[a + 1] < c.cd[a]) c.swap(a, a + 1);
+    }
+    r.cut = r.reach(mabs);
+    if (COUNT && lane == 0) {
+      atomicAdd(&S.st->sdf_cnt[0], c_nodes);
+      atomicAdd(&S.st->sdf_cnt[1], c_leaves);
+      atomicAdd(&S.st->sdf_cnt[2], c_tests);
+    }
+    store_nodes<COUNT, TIES>(S, r, lane == 0, o, true, lane);
+    __syncwarp();
+  }
+}
+
+// ---- a block per 8 x 8 x 4 nodes of the lattice of `stride` S (those whose
+// coordinates are not all multiples of 2 S), a warp per patch of 4 x 4 x 2.  A
+// 2 x 2 x 2 group of nodes (8 lanes) shares the eight nodes of the coarser
+// lattice's cell that holds it, whose closest triangles seed its nodes; a
+// node's cut is then near its final value and the rest is certification:
+//   the block walks the octree level by level, one child per thread, then the
+//     leaves' cubes, against its box (puck_reaches): a list of cubes;
+//   each warp passes the list against its patch's box, one cube per lane, and
+//     the cubes left against its 32 nodes' own cuts, one cube per lane and
+//     one node at a time: a queue of (node, cube) pairs;
+//   the lanes take the pairs as they come free and test their triangles by
+//     tri_dist2_fast; a triangle within its node's cut waits at the node's
+//     lane for the exact test and the candidate list.
+constexpr int kPatchWarps = 8;
+constexpr int kFront = 1024;      // octree nodes of a level within reach of a block (more: its nodes are deferred)
+constexpr int kChunk = 128;       // leaves whose cubes are taken at a time
+constexpr int kBlockCubes = 8 * kChunk;
+constexpr int kCubes = 64;        // a warp's cubes: taken 32 at a time, below 32 left plus one step's 32
+constexpr int kQueue = 512;       // a warp's (node, cube) pairs: flushed above kQueue - 32, plus one node's 32
+constexpr int kHits = 8;          // triangles within a node's cut, waiting for the exact test
+template <bool COUNT, bool TIES>
+__global__ void __launch_bounds__(kPatchWarps * 32, 4) sdf_patch_kernel(const __grid_constant__ Search S,
+                                                                        const __grid_constant__ PyrInfo pi,
+                                                                        int stride, int leaf_max) {
+  __shared__ float4 s_bref[8];                            // the block's reference points
+  __shared__ float4 s_ref[kPatchWarps][8];                // the patches'
+  __shared__ float4 s_node[kPatchWarps][32];              // node position and cut (of the fast distances)
+  __shared__ unsigned s_leaf[kFront];                     // the block's walk: even levels, the leaves last
+  union Walk {
+    unsigned front[kFront];                               // odd levels
+    unsigned short queue[kPatchWarps][kQueue];            // then the warps' pairs: node << 11 | block cube
+  };
+  __shared__ Walk s_w;
+  __shared__ int s_bcube[kBlockCubes];                    // first triangle
+  __shared__ int s_hit[kPatchWarps][kHits][32];
+  __shared__ int s_nhit[kPatchWarps][32];
+  __shared__ int s_seed[kPatchWarps][32];                 // per group: the closest triangles of its cell's corners
+  __shared__ unsigned short s_hq[kPatchWarps][kHits][32]; // the hits' distances, the top half of the float
+  __shared__ unsigned short s_cube[kPatchWarps][kCubes];  // block cubes
+  __shared__ unsigned char s_fmask[2][kFront];
+  __shared__ unsigned char s_bcnt[kBlockCubes];
+  __shared__ int s_off[12], s_dim[12], s_num[13];
+  __shared__ unsigned s_has;
+  static_assert(kBlockCubes <= 2048, "pairs hold 11 bits of cube");
+  const int tid = threadIdx.x;
+  if (tid < 12) {
+    s_off[tid] = (int)pi.off[tid];
+    s_dim[tid] = pi.dim[tid];
+  }
+  if (tid < 13) s_num[tid] = 0;   // per level: the front's nodes; 12: the cubes
+  if (tid == 0) s_has = 0u;
+  __syncthreads();
+  const int n = S.n;
+  const int w = tid >> 5, lane = tid & 31, grp = lane >> 3, sub = lane & 7;
+  const unsigned below = (1u << lane) - 1u;
+  const int nl = (n + stride - 1) / stride;
+  const int ntx = (nl + 7) / 8;
+  const int bx = blockIdx.x % ntx, by = (blockIdx.x / ntx) % ntx;
+  // the middle slabs first: the blocks with the most candidates lie inside the
+  // body, and what runs last should be short
+  const int zq = blockIdx.x / (ntx * ntx), nz = gridDim.x / (ntx * ntx);
+  const int bz = nz / 2 + ((zq & 1) ? -((zq + 1) >> 1) : (zq >> 1));
+  const int i = stride * (bx * 8 + 4 * (w & 1) + 2 * (grp & 1) + (sub & 1));
+  const int j = stride * (by * 8 + 4 * ((w >> 1) & 1) + 2 * (grp >> 1) + ((sub >> 1) & 1));
+  const int k = stride * (bz * 4 + 2 * (w >> 2) + (sub >> 2));
+  const bool here = i < n && j < n && k < n;
+  const bool valid = here && ((i | j | k) & stride);
+  const unsigned vmask = __ballot_sync(0xffffffffu, valid);
+  const int64_t o = lin3(i, j, k, n);
+  // positions past the grid's edge only place the boxes
+  auto pos = [&](int a, int q) { return q < n ? S.axis[a * n + q] : S.axis[a * n + n - 1] + (float)(q - n + 1) * S.h; };
+  const float3 p = make_float3(pos(0, i), pos(1, j), pos(2, k));
+  const float mabs = TIES ? kTieAbs * S.coord : 0.f, h2 = S.h * S.h;
+  Cands<TIES> c;
+  c.init(valid);
+  int bt = -1;
+  unsigned c_tests = 0;
+  // waiting triangles that a later, nearer one has put out of reach leave
+  // their slots
+  auto drop_hits = [&]() {
+    const int mine = min(s_nhit[w][lane], kHits);
+    const float cut = s_node[w][lane].w;
+    int kept = 0;
+#pragma unroll
+    for (int q = 0; q < kHits; ++q) {
+      if (q < mine) {
+        const unsigned short hq = s_hq[w][q][lane];
+        if (__uint_as_float((unsigned)hq << 16) < cut) {
+          s_hit[w][kept][lane] = s_hit[w][q][lane];
+          s_hq[w][kept][lane] = hq;
+          ++kept;
+        }
+      }
+    }
+    s_nhit[w][lane] = kept;
+    return kept;
+  };
+  // the waiting triangles into the candidate lists
+  auto run_hits = [&]() {
+    const int mine = drop_hits();
+    const int most = __reduce_max_sync(0xffffffffu, mine);
+#pragma unroll 1
+    for (int q = 0; q < most; ++q) {
+      if (q < mine) c.offer(p, s_hit[w][q][lane], S, &s_seed[w][8 * grp]);
+    }
+    s_nhit[w][lane] = 0;
+    __syncwarp();
+  };
+  {
+    // seeds: lane `sub` of a group reads the closest triangle of its corner of
+    // the coarser lattice's cell; each distinct one is tested once, for the
+    // node's first cut (within which its cube finds it again)
+    const int s2 = 2 * stride;
+    const int ci = (i & ~(s2 - 1)) + s2 * (sub & 1), cj = (j & ~(s2 - 1)) + s2 * ((sub >> 1) & 1),
+              ck = (k & ~(s2 - 1)) + s2 * (sub >> 2);
+    int t = -1;
+    if (ci < n && cj < n && ck < n) t = S.seed_ids[lin3(ci, cj, ck, n)];
+    const unsigned same = __match_any_sync(0xffffffffu, t) & (0xffu << (8 * grp));
+    unsigned left = (__ballot_sync(0xffffffffu, t >= 0 && lane == __ffs(same) - 1) >> (8 * grp)) & 0xffu;
+    float bq = INFINITY;
+    while (__any_sync(0xffffffffu, left != 0u)) {
+      const int tq = __shfl_sync(0xffffffffu, t, left ? 8 * grp + __ffs(left) - 1 : lane);
+      if (here && left != 0u) {
+        const float q = tri_dist2_fast(p, S.tris_s + kTriRec * (int64_t)tq);
+        if (q < bq) {
+          bq = q;
+          bt = tq;
+        }
+      }
+      left &= left - 1u;
+    }
+    s_nhit[w][lane] = 0;
+    s_seed[w][lane] = t;
+    s_node[w][lane] = make_float4(p.x, p.y, p.z, !valid ? -INFINITY : bt < 0 ? INFINITY : fast_cut(bq, mabs, h2));
+  }
+  // the boxes of the patch and of the block: half extents (plus the rounding
+  // of the positions), centres, and reference points: the closest points of
+  // their eight corner nodes (a corner past the grid's edge takes another's)
+  const float eg = 0.5f * (float)stride * S.h * (1.f + 1e-5f) + 2e-7f * S.coord;
+  const float3 ep = make_float3(3.f * eg, 3.f * eg, eg), eb = make_float3(7.f * eg, 7.f * eg, 3.f * eg);
+  const float epl = 4.3588995f * eg, ebl = 10.344085f * eg;   // sqrt(19), sqrt(107)
+  auto mid = [&](float v) {
+    return 0.5f * (__shfl_sync(0xffffffffu, v, 0) + __shfl_sync(0xffffffffu, v, 31));
+  };
+  const float3 pp = make_float3(mid(p.x), mid(p.y), mid(p.z));
+  const float3 pb = make_float3(0.5f * (pos(0, stride * 8 * bx) + pos(0, stride * (8 * bx + 7))),
+                                0.5f * (pos(1, stride * 8 * by) + pos(1, stride * (8 * by + 7))),
+                                0.5f * (pos(2, stride * 4 * bz) + pos(2, stride * (4 * bz + 3))));
+  const unsigned with = __ballot_sync(0xffffffffu, here && bt >= 0);
+  {
+    // corner q of a patch: the node of group (q & 3) at the same corner; the
+    // block's corner w lies at the corner w of its patch w
+    const int cl = 8 * (lane & 3) + (lane & 7);
+    const int ref = (with >> cl) & 1u ? cl : 31 - __clz(with | 1u);
+    const float3 rp = make_float3(__shfl_sync(0xffffffffu, p.x, ref), __shfl_sync(0xffffffffu, p.y, ref),
+                                  __shfl_sync(0xffffffffu, p.z, ref));
+    const int rt = __shfl_sync(0xffffffffu, bt, ref);
+    if (lane < 8 && with != 0u) {
+      const float3 y = closest_on(rp, S.tris_s + kTriRec * (int64_t)rt);
+      s_ref[w][lane] = make_float4(y.x, y.y, y.z, reach_of(pp, y, epl, S.coord));
+      if (lane == w) {
+        s_bref[w] = make_float4(y.x, y.y, y.z, reach_of(pb, y, ebl, S.coord));
+        atomicOr(&s_has, 1u << w);
+      }
+    }
+  }
+  // the walk begins at the first level of at most 4 nodes per axis
+  int l0 = pi.nlev - 1;
+  while (l0 > 1 && s_dim[l0 - 1] <= 4) --l0;
+  if (tid < s_dim[l0] * s_dim[l0] * s_dim[l0]) {
+    const int d = s_dim[l0];
+    const int z = tid / (d * d), r = tid - z * d * d, y = r / d, x = r - y * d;
+    const float rad = S.pyr[2 * (int64_t)(s_off[l0] + tid)].w;
+    (l0 & 1 ? s_w.front : s_leaf)[tid] = ((unsigned)z << 18) | ((unsigned)y << 9) | (unsigned)x;
+    s_fmask[l0 & 1][tid] = rad < 0.f ? 0 : (unsigned char)(__float_as_uint(rad) & 0xffu);   // empty: no children
+    if (tid == 0) s_num[l0] = d * d * d;
+  }
+  __syncthreads();
+  const unsigned has = s_has;
+  if (has != 0xffu && has != 0u) {   // a patch without nodes leaves its corner to another's reference
+    if (tid < 8 && !((has >> tid) & 1u)) s_bref[tid] = s_bref[__ffs(has) - 1];
+    __syncthreads();
+  }
+  bool heavy = false;
+  int m = 0;
+  if (has != 0u) {
+    // the octree, a level at a time; level 0 are the leaves (their indices)
+    for (int lev = l0; lev > 0; --lev) {
+      m = s_num[lev];
+      if (m > kFront) break;
+      const unsigned* cur = lev & 1 ? s_w.front : s_leaf;
+      unsigned* nxt = lev & 1 ? s_leaf : s_w.front;
+      const int dc = s_dim[lev - 1];
+      for (int b0 = 0; b0 < 8 * m; b0 += kPatchWarps * 32) {
+        const int q = b0 + tid, ch = q & 7;
+        bool keep = false;
+        unsigned cm = 0, ent = 0;
+        if (q < 8 * m && (s_fmask[lev & 1][q >> 3] >> ch) & 1u) {
+          const unsigned e = cur[q >> 3];
+          const int cx = 2 * (int)(e & 511u) + (ch & 1), cy = 2 * (int)((e >> 9) & 511u) + ((ch >> 1) & 1),
+                    cz = 2 * (int)(e >> 18) + (ch >> 2);
+          const int64_t cg = s_off[lev - 1] + ((int64_t)cz * dc + cy) * dc + cx;
+          const float4 A = S.pyr[2 * cg];
+          keep = puck_reaches<8>(pb, s_bref, eb, ebl, A, S.pyr[2 * cg + 1]);
+          cm = __float_as_uint(A.w) & 0xffu;
+          ent = lev == 1 ? (unsigned)leaf_index(cx, cy, cz, S.nb)
+                         : ((unsigned)cz << 18) | ((unsigned)cy << 9) | (unsigned)cx;
+        }
+        const unsigned b = __ballot_sync(0xffffffffu, keep);
+        int at = 0;
+        if (lane == 0 && b) at = atomicAdd(&s_num[lev - 1], __popc(b));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & below);
+        if (keep && at < kFront) {
+          nxt[at] = ent;
+          s_fmask[(lev & 1) ^ 1][at] = (unsigned char)cm;
+        }
+      }
+      __syncthreads();
+      m = s_num[lev - 1];
+    }
+    heavy = m > leaf_max;
+  }
+  if (heavy) {
+    if (!vmask) return;
+    unsigned base = 0;
+    if (lane == 0) base = atomicAdd(&S.st->ndefer, (unsigned)__popc(vmask));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (valid) {
+      S.defer[base + __popc(vmask & below)] = (int)o;
+      S.seed_ids[o] = bt;
+    }
+    return;
+  }
+  int ncube = 0, nq = 0;
+  unsigned short* queue = s_w.queue[w];
+  // the queued pairs' triangles, a lane taking the next pair when it is
+  // through with one
+  auto run_queue = [&]() {
+    __syncwarp();
+    int next = 0, t = 0, t1 = 0, v = 0;
+    float3 x = p;
+    while (true) {
+      const unsigned free = __ballot_sync(0xffffffffu, t == t1);
+      if (t == t1) {
+        const int at = next + __popc(free & below);
+        if (at < nq) {
+          const unsigned e = queue[at];
+          v = (int)(e >> 11);
+          t = s_bcube[e & 2047u];
+          t1 = t + s_bcnt[e & 2047u];
+          x = f3(s_node[w][v]);
+        }
+      }
+      next += __popc(free);
+      const bool on = t < t1;
+      if (!__any_sync(0xffffffffu, on)) break;
+      if (COUNT) c_tests += (unsigned)__popc(__ballot_sync(0xffffffffu, on));
+      bool hit = false;
+      float q = 0.f;
+      const int tq = t;
+      if (on) {
+        q = tri_dist2_fast(x, S.tris_s + kTriRec * (int64_t)t);
+        hit = q < *reinterpret_cast<volatile float*>(&s_node[w][v].w);
+        ++t;
+      }
+      while (__any_sync(0xffffffffu, hit)) {
+        if (hit) {
+          atomicMin(reinterpret_cast<int*>(&s_node[w][v].w), __float_as_int(fast_cut(q, mabs, h2)));
+          const int at = atomicAdd(&s_nhit[w][v], 1);
+          if (at < kHits) {
+            s_hit[w][at][v] = tq;
+            s_hq[w][at][v] = (unsigned short)(__float_as_uint(q) >> 16);
+            hit = false;
+          }
+        }
+        if (__any_sync(0xffffffffu, hit)) {   // a node's slots are full
+          __syncwarp();
+          if (__any_sync(0xffffffffu, drop_hits() > kHits - 2)) run_hits();
+          __syncwarp();
+        }
+      }
+    }
+    nq = 0;
+    __syncwarp();
+  };
+  // up to 32 listed cubes against each node's own cut
+  auto run_cubes = [&](bool last) {
+    const int take = min(ncube, 32);
+    ncube -= take;
+    const bool done = last && ncube == 0;
+    // 16 cubes or fewer: two lanes share a cube, each with half of the nodes
+    const bool halves = take <= 16;
+    const int at0 = halves ? lane & 15 : lane;
+    const int bi = at0 < take ? s_cube[w][ncube + at0] : 0;
+    const int64_t q0 = s_bcube[bi];
+    const float4 A = S.cell_pyr[2 * q0], B = S.cell_pyr[2 * q0 + 1];
+    unsigned mine = 0;   // the cube's nodes
+    const int v0 = halves ? lane & 16 : 0, v1 = halves ? 16 : 32;
+#pragma unroll 8
+    for (int v = 0; v < v1; ++v) {
+      const float4 nd = s_node[w][v0 + v];
+      if (puck_dist2(f3(nd), A, B) < nd.w) mine |= 1u << v;
+    }
+    mine = mine << v0;
+    if (at0 >= take) mine = 0;
+    // the pairs, cube by cube (the lanes that take them share triangles); what
+    // does not fit waits for the queue to be worked off
+    while (true) {
+      int at = __popc(mine);   // inclusive prefix sum over the lanes
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, at, d);
+        if (lane >= d) at += x;
+      }
+      const int all = __shfl_sync(0xffffffffu, at, 31);
+      at += nq - __popc(mine);
+      while (mine != 0u && at < kQueue) {
+        queue[at++] = (unsigned short)(((__ffs(mine) - 1) << 11) | bi);
+        mine &= mine - 1u;
+      }
+      nq = min(nq + all, kQueue);
+      const bool more = __any_sync(0xffffffffu, mine != 0u);
+      if (more || done) run_queue();
+      if (!more) break;
+    }
+    __syncwarp();
+  };
+  for (int c0 = 0; c0 < m; c0 += kChunk) {
+    if (c0 > 0) {
+      __syncthreads();
+      if (tid == 0) s_num[12] = 0;
+      __syncthreads();
+    }
+    const int leaves = min(m - c0, kChunk);
+    for (int b0 = 0; b0 < 8 * leaves; b0 += kPatchWarps * 32) {
+      const int q = b0 + tid;
+      int q0 = 0, cnt = 0;
+      if (q < 8 * leaves) leaf_cube(S, (int)s_leaf[c0 + (q >> 3)], q & 7, q0, cnt);
+      const bool in = cnt > 0 && puck_reaches<8>(pb, s_bref, eb, ebl, S.cell_pyr[2 * (int64_t)q0],
+                                                 S.cell_pyr[2 * (int64_t)q0 + 1]);
+      const unsigned b = __ballot_sync(0xffffffffu, in);
+      int at = 0;
+      if (lane == 0 && b) at = atomicAdd(&s_num[12], __popc(b));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & below);
+      if (in) {
+        s_bcube[at] = q0;
+        s_bcnt[at] = (unsigned char)cnt;
+      }
+    }
+    __syncthreads();
+    if (!vmask) continue;
+    const int nbc = s_num[12];
+    for (int b0 = 0; b0 < nbc; b0 += 32) {
+      const int q = b0 + lane;
+      bool in = false;
+      if (q < nbc) {
+        const int64_t q0 = s_bcube[q];
+        in = puck_reaches<4>(pp, s_ref[w], ep, epl, S.cell_pyr[2 * q0], S.cell_pyr[2 * q0 + 1]);
+      }
+      const unsigned b = __ballot_sync(0xffffffffu, in);
+      if (in) s_cube[w][ncube + __popc(b & below)] = (unsigned short)q;
+      ncube += __popc(b);
+      __syncwarp();
+      const bool last = b0 + 32 >= nbc;
+      while (ncube >= 32 || (last && (ncube > 0 || nq > 0))) run_cubes(last);
+    }
+  }
+  if (!vmask) return;
+  run_hits();
+  if (COUNT && lane == 0) {
+    if (w == 0) {
+      for (int l = 1; l < pi.nlev; ++l) atomicAdd(&S.st->sdf_cnt[0], (unsigned long long)s_num[l]);
+      atomicAdd(&S.st->sdf_cnt[1], (unsigned long long)m);
+    }
+    atomicAdd(&S.st->sdf_cnt[2], (unsigned long long)c_tests);
+  }
+  c.cut = c.reach(mabs);
+  store_nodes<COUNT, TIES>(S, c, valid, o, stride > 1, lane);
+}
+
+// Float-float decision between the float32 near-tie candidates of a node:
+// distances (tri_dist2_ff_exact on the ~48-bit vertices) from the node position
+// rounded once from double, the smaller wins; equal distances (a shared edge or
+// vertex: the same closest point) take the smaller triangle index.  The node
+// coordinates come from per-axis float-float tables built once per block, and
+// chi >= c (c double) is tested as chi >= the smallest float not below c, so no
+// node needs FP64.
+//
+// Candidates of one class (the top 32 - id_bits bits of feature_class; id_bits
+// 0: none) are not told apart here: the float32 distance, and where that is
+// equal the order of the candidate list, decides between them beforehand.  The nodes' results
+// have always been those of this rule (one pair of features in 2^(32 -
+// id_bits)), and a node between two triangles whose vertices are sensitive can
+// carry 5e-5 of a dense gradient's norm to one or the other.  The
+// seeds are the triangles of the stride-2 lattice around the node.  The nodes of that lattice (even != 0) take their
+// own pass, after the others have read their triangles.
+__global__ void sdf_tie_kernel(const __grid_constant__ Search S, SurfParams g, int id_bits, int even) {
   __shared__ float2 s_ax[3][kMaxRes];
   const int n = g.res;
   for (int t = threadIdx.x; t < 3 * n; t += blockDim.x) {
@@ -1404,40 +2044,70 @@ __global__ void sdf_tie_kernel(const float* __restrict__ chi, SurfParams g, cons
     s_ax[a][i] = make_float2(hi, (float)(v - (double)hi));
   }
   __syncthreads();
-  const float cf = st->c_up;
+  const float cf = S.st->c_up;
   const unsigned un = (unsigned)n;
-  const unsigned count = st->ntie;
-  const int xi = st->fwd.xidx ^ 1;
+  const unsigned count = S.st->ntie;
+  const int xi = S.st->fwd.xidx ^ 1;
   for (unsigned it = blockIdx.x * blockDim.x + threadIdx.x; it < count; it += gridDim.x * blockDim.x) {
-    const unsigned o = (unsigned)tie_list[it];
-    const int t1 = tie_b[it];
-    const int t0 = tie_a[it];
-    const int2 t23 = tie_cd.p[xi][it];
+    const unsigned o = (unsigned)S.tie_list[it];
     const unsigned row = o / un;
     const int i = (int)(o - row * un), j = (int)(row % un), k = (int)(row / un);
+    if ((((i | j | k) & 1) == 0) != (even != 0)) continue;
+    const int2 t23 = S.tie_cd.p[xi][it];
+    int cand[kCand] = {S.tie_a[it], S.tie_b[it], t23.x, t23.y};
     const float2 px = s_ax[0][i], py = s_ax[1][j], pz = s_ax[2][k];
+    const float3 p = make_float3(px.x, py.x, pz.x);
+    int left = 0;
+    if (id_bits > 0) {
+      float d2[kCand];
+      unsigned cls[kCand];
+#pragma unroll 1
+      for (int q = 0; q < kCand; ++q) {
+        if (cand[q] < 0) continue;
+        float v, w;
+        d2[q] = tri_dist2_rec(p, S.tris_s + kTriRec * (int64_t)cand[q], v, w);
+        cls[q] = feature_class(v, w, S.tris, cand[q]) >> id_bits;
+        for (int r = 0; r < q && cand[q] >= 0; ++r) {
+          if (cand[r] < 0 || cls[r] != cls[q]) continue;
+          bool stays = d2[r] < d2[q];
+          if (d2[r] == d2[q]) {
+            int seeds[8];
+            for (int c = 0; c < 8; ++c) {
+              const int ci = (i & ~1) + 2 * (c & 1), cj = (j & ~1) + 2 * ((c >> 1) & 1), ck = (k & ~1) + 2 * (c >> 2);
+              seeds[c] = !even && ci < n && cj < n && ck < n ? S.ctri[lin3(ci, cj, ck, n)] : -1;
+            }
+            stays = comes_first(cand[r], cand[q], S.tris_lo, seeds);
+          }
+          cand[stays ? q : r] = -1;
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kCand; ++q) left += cand[q] >= 0;
     const Vec3<Ff> pf = {Ff(px.x, px.y), Ff(py.x, py.y), Ff(pz.x, pz.y)};
     Ff bd(INFINITY);
     int bi = -1;
-    const int cand[kCand] = {t0, t1, t23.x, t23.y};
     // one copy of the float-float distance in the loop: unrolled, the four
     // copies overflow the instruction cache
 #pragma unroll 1
     for (int q = 0; q < kCand; ++q) {
       if (cand[q] < 0) continue;
-      const Ff d2 = tris_lo ? tri_dist2_ff_exact(pf, tris_s + kTriRec * (int64_t)cand[q], tris[cand[q]],
-                                                 tris_lo[cand[q]])
-                            : tri_dist2_rec_ff(pf, tris_s + kTriRec * (int64_t)cand[q]);
+      if (left == 1) {   // decided by its class: the distance stays the search's
+        bi = cand[q];
+        break;
+      }
+      const Ff d2 = tri_dist2_ff_exact(pf, S.tris_s + kTriRec * (int64_t)cand[q], S.tris[cand[q]], S.tris_lo[cand[q]]);
       if (bi < 0 || d2 < bd || (!(bd < d2) && cand[q] < bi)) {
         bd = d2;
         bi = cand[q];
       }
     }
-    const float sgn = (chi[o] >= cf) ? 1.f : -1.f;
+    S.ctri[o] = bi;
+    if (left == 1) continue;
+    const float sgn = (S.chi[o] >= cf) ? 1.f : -1.f;
     const float val = sgn * sqrtf(__fadd_rn(bd.hi, bd.lo));
-    phi[o] = val;
-    if (sdf_out) sdf_out[o] = val;
-    ctri[o] = bi;
+    S.phi[o] = val;
+    if (S.sdf_out) S.sdf_out[o] = val;
   }
 }
 
@@ -1910,7 +2580,7 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
   }
   int rc = exclusive_scan(h->brick_count, h->brick_off, nbricks, h->scan_tmp, s);
   if (rc) return rc;
-  mc_total_kernel<<<1, 1, 0, s>>>(h->brick_off, nbricks, h->mesh_cap, h->leaf_off, h->dstate);
+  mc_total_kernel<<<1, 256, 0, s>>>(h->brick_off, nbricks, h->mesh_cap, h->leaf_off, h->dstate, g, h->axis);
   WGEO_LAUNCH_CHECK();
   // the bricks with triangles, listed in the solver's idle residual buffer
   int* live_bricks = reinterpret_cast<int*>(h->r32);
@@ -1961,61 +2631,105 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
   stage_end(h, kStMC, slot, s);
   slot = stage_begin(h, kStSDF, s);
   // the solver's residual / correction scratch is idle until the next solve:
-  // it holds the near-tie candidates between the two kernels
-  int* tie_a = reinterpret_cast<int*>(h->r32);
-  int* tie_b = reinterpret_cast<int*>(h->e32);
-  // ... and so does the float-float iterate buffer that is not the current one
-  // (its index is on the device): two more candidates per node
-  TieSlots tie_cd;
-  tie_cd.p[0] = reinterpret_cast<int2*>(h->chiff[0]);
-  tie_cd.p[1] = reinterpret_cast<int2*>(h->chiff[1]);
-  int* ctri = h->opt.keep_for_backward ? h->ctri : nullptr;
-  // closest triangles of the coarser passes, read by the finer ones as seeds
-  int* seed_ids = ctri ? ctri : tie_a;
-  // the near-tie list: nodes re-decided by the tie pass, in the adjoint's
+  // it holds the near-tie candidates between the two kernels, and so does the
+  // float-float iterate buffer that is not the current one (its index is on
+  // the device); the near-tie list and the deferred nodes lie in the adjoint's
   // dL/dchi buffer, which is idle until a backward clears it
-  int* tie_list = ctri ? reinterpret_cast<int*>(h->dchi64) : nullptr;
-  if (ctri) WGEO_CUDA_TRY(cudaMemsetAsync(&h->dstate->ntie, 0, sizeof(unsigned), s));
-  // closest-feature keys of the near-tie candidates: the bits above the
-  // triangle ids (ids < cap <= 2^id_bits - 1; at least 8 key bits)
-  int id_bits = 0;
-  if (ctri) {
-    while (id_bits < 32 && ((int64_t)1 << id_bits) - 1 < h->mesh_cap) ++id_bits;
-    if (id_bits > 24) id_bits = 0;
-  }
-  for (int stride = kSdfCoarse; stride >= 1; stride /= 2) {
-    const int nl = (res + stride - 1) / stride;
-    const int nblk = ((nl + 7) / 8) * ((nl + 7) / 8) * ((nl + 1) / 2);
+  const int64_t N = (int64_t)res * res * res;
+  int* ctri = h->opt.keep_for_backward ? h->ctri : nullptr;
+  Search S;
+  S.tris_s = h->tris_s;
+  S.tris = h->tris;
+  S.tris_lo = h->tris_lo;
+  S.leaf_off = h->leaf_off;
+  S.leaf_cnt = h->leaf_cnt;
+  S.pyr = h->pyramid;
+  S.cell_pyr = h->cell_pyr;
+  S.axis = h->axis;
+  S.chi = h->chi32;
+  S.st = h->dstate;
+  S.cap = h->mesh_cap;
+  S.n = res;
+  S.nb = g.nb;
+  S.h = (float)g.h;
+  S.coord = 0.f;
+  for (int a = 0; a < 3; ++a)
+    S.coord = std::max(S.coord, (float)std::max(fabs(g.lo[a]), fabs(g.lo[a] + res * g.h)));
+  S.phi = h->phi;
+  S.sdf_out = sdf_out;
+  S.ctri = ctri;
+  S.tie_a = reinterpret_cast<int*>(h->r32);
+  S.tie_b = reinterpret_cast<int*>(h->e32);
+  S.tie_cd.p[0] = reinterpret_cast<int2*>(h->chiff[0]);
+  S.tie_cd.p[1] = reinterpret_cast<int2*>(h->chiff[1]);
+  S.tie_list = ctri ? reinterpret_cast<int*>(h->dchi64) : nullptr;
+  S.defer = ctri ? S.tie_list + N : S.tie_b;
+  // closest triangles of the coarser lattices, read by the finer ones as seeds
+  S.seed_ids = ctri ? ctri : S.tie_a;
+  static_assert(offsetof(DevState, ndefer) == offsetof(DevState, ntie) + sizeof(unsigned), "cleared together");
+  WGEO_CUDA_TRY(cudaMemsetAsync(&h->dstate->ntie, 0, 2 * sizeof(unsigned), s));
+  const bool count = h->opt.stage_timing == 2;
+  const int threads = kWarps * 32;
+  auto node_pass = [&](bool list, int stride) -> int {
+    const int64_t nl = (res + stride - 1) / stride;
+    const int blocks = list ? h->num_sms * 8 : grid_blocks(32 * nl * nl * nl, threads, h->num_sms * 64);
+#define WGEO_NODE_PASS(C, T)                                                          \
+  if (list)                                                                           \
+    sdf_node_kernel<C, T, true><<<blocks, threads, 0, s>>>(S, pi, stride);            \
+  else                                                                                \
+    sdf_node_kernel<C, T, false><<<blocks, threads, 0, s>>>(S, pi, stride);
     if (ctri) {
-      if (h->opt.stage_timing == 2)
-        sdf_kernel<true, true><<<nblk, kWarps * 32, 0, s>>>(h->chi32, g, h->dstate, h->tris_s, id_bits, h->leaf_off,
-                                                            h->mesh_cap, h->pyramid, pi, h->phi, sdf_out, ctri,
-                                                            tie_a, tie_b, tie_cd, tie_list, seed_ids, stride,
-                                                            h->leaf_cnt, h->cell_pyr);
-      else
-        sdf_kernel<false, true><<<nblk, kWarps * 32, 0, s>>>(h->chi32, g, h->dstate, h->tris_s, id_bits, h->leaf_off,
-                                                             h->mesh_cap, h->pyramid, pi, h->phi, sdf_out, ctri,
-                                                             tie_a, tie_b, tie_cd, tie_list, seed_ids, stride,
-                                                            h->leaf_cnt, h->cell_pyr);
+      if (count) { WGEO_NODE_PASS(true, true) } else { WGEO_NODE_PASS(false, true) }
     } else {
-      if (h->opt.stage_timing == 2)
-        sdf_kernel<true, false><<<nblk, kWarps * 32, 0, s>>>(h->chi32, g, h->dstate, h->tris_s, id_bits, h->leaf_off,
-                                                             h->mesh_cap, h->pyramid, pi, h->phi, sdf_out, nullptr,
-                                                             nullptr, nullptr, tie_cd, nullptr, seed_ids, stride,
-                                                             h->leaf_cnt, h->cell_pyr);
+      if (count) { WGEO_NODE_PASS(true, false) } else { WGEO_NODE_PASS(false, false) }
+    }
+#undef WGEO_NODE_PASS
+    WGEO_LAUNCH_CHECK();
+    return WGEO_OK;
+  };
+  // stride of the coarsest lattice.  A coarser one costs fewer searches from
+  // nothing (4,300 warp instructions a node at 128^3, 7,200 at 256^3), but its
+  // patch passes have too few blocks to fill the chip and boxes with many
+  // candidates.  Search stage at 64^3 / 128^3 / 256^3 / 512^3, ms: stride 2
+  // 0.32 / - / - / -, 4 0.37 / 1.70 / 11.8 / 102, 8 0.47 / 2.05 / 11.5 / 85, 16
+  // at 512^3 94.
+  const int coarse = res <= 80 ? 2 : res <= 160 ? 4 : 8;
+  rc = node_pass(false, coarse);
+  if (rc) return rc;
+  for (int stride = coarse / 2; stride >= 1; stride /= 2) {
+    const int nl = (res + stride - 1) / stride;
+    const int nblk = ((nl + 7) / 8) * ((nl + 7) / 8) * ((nl + 3) / 4);
+    // leaves in a block's reach above which its nodes are searched one by one:
+    // cheaper in a block (a third of the instructions), but where the blocks
+    // are few the longest decides.  Search stage at 256 / 512 / 1024, ms: 0.29 /
+    // 0.38 / 0.53 on a 64^3 sphere (every triangle is in reach of its centre),
+    // 1.76 / 1.57 / 1.68 at 128^3, 14.2 / 11.5 / 10.8 at 256^3.
+    const int leaf_max = res <= 80 ? 256 : nblk <= 16384 ? 512 : kFront;
+    if (ctri) {
+      if (count)
+        sdf_patch_kernel<true, true><<<nblk, kPatchWarps * 32, 0, s>>>(S, pi, stride, leaf_max);
       else
-        sdf_kernel<false, false><<<nblk, kWarps * 32, 0, s>>>(h->chi32, g, h->dstate, h->tris_s, id_bits, h->leaf_off,
-                                                              h->mesh_cap, h->pyramid, pi, h->phi, sdf_out, nullptr,
-                                                              nullptr, nullptr, tie_cd, nullptr, seed_ids, stride,
-                                                             h->leaf_cnt, h->cell_pyr);
+        sdf_patch_kernel<false, true><<<nblk, kPatchWarps * 32, 0, s>>>(S, pi, stride, leaf_max);
+    } else {
+      if (count)
+        sdf_patch_kernel<true, false><<<nblk, kPatchWarps * 32, 0, s>>>(S, pi, stride, leaf_max);
+      else
+        sdf_patch_kernel<false, false><<<nblk, kPatchWarps * 32, 0, s>>>(S, pi, stride, leaf_max);
     }
     WGEO_LAUNCH_CHECK();
   }
+  rc = node_pass(true, 1);
+  if (rc) return rc;
   stage_end(h, kStSDF, slot, s);
   if (ctri) {
     slot = stage_begin(h, kStSDFTie, s);
-    sdf_tie_kernel<<<152 * 8, 256, 0, s>>>(h->chi32, g, h->dstate, h->tris_s, h->tris, h->tris_lo, tie_a, tie_b,
-                                           tie_cd, tie_list, h->phi, sdf_out, ctri);
+    // bits of a triangle id (ids < cap <= 2^id_bits - 1; at most 24)
+    int id_bits = 0;
+    while (id_bits < 32 && ((int64_t)1 << id_bits) - 1 < h->mesh_cap) ++id_bits;
+    if (id_bits > 24) id_bits = 0;
+    sdf_tie_kernel<<<152 * 8, 256, 0, s>>>(S, g, id_bits, 0);
+    WGEO_LAUNCH_CHECK();
+    sdf_tie_kernel<<<152 * 8, 256, 0, s>>>(S, g, id_bits, 1);
     WGEO_LAUNCH_CHECK();
     stage_end(h, kStSDFTie, slot, s);
   }

@@ -60,6 +60,7 @@ struct DevState {
                                    // nodes re-decided in float-float
   unsigned nsliver;                // backward: nodes whose closest triangle is a sliver (FP64 pass)
   unsigned ntie;                   // forward: nodes on the near-tie list (distance search)
+  unsigned ndefer;                 // forward: nodes left to the search's per-node pass (cleared with ntie)
   unsigned splat_tiles;            // forward: splat tiles with a point in reach (the active list)
   unsigned splat_next;             // forward: next active tile to be taken by a splat CTA
   unsigned nleaf_live;             // forward: octree leaves holding triangles (the live list)
@@ -245,14 +246,14 @@ __device__ __forceinline__ bool operator<=(Ff a, Ff b) { return !(b < a); }
 __device__ __forceinline__ bool operator>=(Ff a, Ff b) { return !(a < b); }
 
 // Closest-point weights (v, w) of y = a + v ab + w ac on a triangle given by
-// its search record (r0 = (a, |ab|^2), r1 = (ab, vertex keys), r2 = (ac, |ac|^2),
+// its search record (r0 = (a, |ab|^2), r1 = (ab, ab.ac), r2 = (ac, |ac|^2),
 // r3 = (1/|ab|^2, 1/|ac|^2, 1/|bc|^2, 1/|ab x ac|^2)), from ap = p - a,
 // d1 = ab.ap and d2 = ac.ap: Ericson's Voronoi-region case analysis with the
 // six dot products reduced to two through the Gram entries and the
 // divisions replaced by the reciprocals.
 __device__ __forceinline__ void rec_weights(const float3 ap, float d1, float d2, const float4 r0, const float4 r1,
                                             const float4 r2, const float4 r3, float& v, float& w) {
-  const float e00 = r0.w, e01 = r1.x * r2.x + r1.y * r2.y + r1.z * r2.z, e11 = r2.w;   // r1.w: vertex keys
+  const float e00 = r0.w, e01 = r1.w, e11 = r2.w;
   const float d3 = d1 - e00, d4 = d2 - e01;                  // ab . bp, ac . bp
   const float d5 = d1 - e01, d6 = d2 - e11;                  // ab . cp, ac . cp
   if (d1 <= 0.f && d2 <= 0.f) {
@@ -413,6 +414,8 @@ struct wgeo_handle {
   int* tile_count = nullptr;
   int* tile_off = nullptr;       // ntiles + 1
   int* tile_cursor = nullptr;
+
+  float* axis = nullptr;         // node coordinates of the last forward, [3][res]
 
   // mesh
   int64_t mesh_cap = 0;
