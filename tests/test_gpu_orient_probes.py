@@ -1,0 +1,48 @@
+"""Ray probes of the orientation pass where a batch's points fall on few probes
+(shared by the warp), on all of them (one lane each), or on both in turn, and
+where the largest nearest-neighbour gap belongs to one far point: integer
+decisions, equal to the oracle's."""
+import numpy as np
+import pytest
+
+from oracle import orient as O
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+BOX = np.array([0, 0, 0, 1, 1, 1], dtype=np.float32)
+
+
+def _cloud(kind, rng, n):
+    if kind == "volume":         # a few points in every cell
+        return rng.uniform(0.05, 0.95, (n, 3))
+    if kind == "clusters":       # hundreds of points in few cells
+        c = np.array([[0.2, 0.2, 0.2], [0.8, 0.5, 0.5], [0.5, 0.8, 0.3]])
+        return c[rng.integers(0, 3, n)] + rng.uniform(-0.02, 0.02, (n, 3))
+    if kind == "far":            # the same, and one point that sets the radius
+        p = 0.3 + rng.uniform(-0.03, 0.03, (n, 3))
+        p[n // 2] = 0.6
+        return p
+    d = rng.standard_normal((n, 3))
+    return 0.5 + 0.35 * d / np.linalg.norm(d, axis=1, keepdims=True)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 1500])
+@pytest.mark.parametrize("kind", ["volume", "clusters", "far", "sphere"])
+def test_probe_batches_match_the_oracle(kind, n):
+    import __graft_entry__ as g
+    g.build()
+    from paper_2609_20964_gb300 import Reconstructor
+    rng = np.random.default_rng(n)
+    p = _cloud(kind, rng, n).astype(np.float32)
+    d = rng.standard_normal((n, 3))
+    N = (d / np.linalg.norm(d, axis=1, keepdims=True)).astype(np.float32)
+    rec = Reconstructor(16, n)
+    out, st, rd = rec.orient_normals(torch.from_numpy(p).cuda(), torch.from_numpy(N).cuda(), BOX, 2.5, 2,
+                                     with_stats=True)
+    on, os_, ord_ = O.orient(p, N)
+    assert np.float32(rd.item()) == ord_
+    assert np.array_equal(st.cpu().numpy().astype(np.int64), os_)
+    assert np.array_equal(out.cpu().numpy(), on)
+    rec.close()
