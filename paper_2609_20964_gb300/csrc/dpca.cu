@@ -228,6 +228,13 @@ __device__ __forceinline__ float jacobi_min_vector(float a[3][3], float v_out[3]
 // of a point does not depend on the warp's make-up.  rc = R / cell edge plus
 // a margin for the rounding of cell coordinates and of the membership test.
 //
+// Issue of the pair arithmetic bounds the kernel (about 30 instructions an
+// entry, none of them shared between points).  Groups that lie wholly in the
+// row's range, nearly all of them, run a lane's four entries unrolled with the
+// four loads first, the partial ones a plain loop: 2 10^5 points of a sphere at
+// R = 0.1 (about 4600 neighbours) 2831 -> 2390 us, 10^6 at 50 neighbours a disc
+// 1130 -> 1020 (1060 without the bound of 8 blocks an SM on the registers).
+//
 // Weights.  w' = R w = 1 / (d / R + eps / R), at most R / eps <= 1e6, from the
 // hardware square root and reciprocal (relative error ~1e-7; weights decide
 // nothing, they only scale the moments).
@@ -242,7 +249,12 @@ __device__ __forceinline__ float approx_rcp(float x) {
   return y;
 }
 
-__global__ void __launch_bounds__(128, 4) dpca_normal_kernel(const float4* __restrict__ sorted,
+// dx^2 + dy^2 + dz^2, every operation rounded.
+__device__ __forceinline__ float dist2_rn(float dx, float dy, float dz) {
+  return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+}
+
+__global__ void __launch_bounds__(128, 8) dpca_normal_kernel(const float4* __restrict__ sorted,
                                                           const int* __restrict__ off,
                                                           const int* __restrict__ total, PointGrid g,
                                                           const float4* __restrict__ gbox, int* __restrict__ next,
@@ -275,6 +287,28 @@ __global__ void __launch_bounds__(128, 4) dpca_normal_kernel(const float4* __res
     float S0 = 0.f, S1x = 0.f, S1y = 0.f, S1z = 0.f;
     float Sxx = 0.f, Sxy = 0.f, Sxz = 0.f, Syy = 0.f, Syz = 0.f, Szz = 0.f;
     int cnt = 0;
+    auto add = [&](const float4 pj) {   // one entry's terms of the sums
+      float dx = pj.x - q.x, dy = pj.y - q.y, dz = pj.z - q.z;
+      const float d2 = dist2_rn(dx, dy, dz);
+      const bool in = d2 <= r2;
+      dx = in ? dx : 0.f;
+      dy = in ? dy : 0.f;
+      dz = in ? dz : 0.f;
+      const float w = in ? approx_rcp(fmaf(approx_sqrt(d2), inv_r, eps_r)) : 0.f;   // R w
+      const float wu = w * inv_r;
+      const float wx = wu * dx, wy = wu * dy, wz = wu * dz;   // R w y, y = (x_j - x_i) / R
+      S0 += w;
+      S1x += wx;
+      S1y += wy;
+      S1z += wz;
+      Sxx = fmaf(wx, dx, Sxx);   // R^2 w y y^T: one more 1/R below
+      Sxy = fmaf(wx, dy, Sxy);
+      Sxz = fmaf(wx, dz, Sxz);
+      Syy = fmaf(wy, dy, Syy);
+      Syz = fmaf(wy, dz, Syz);
+      Szz = fmaf(wz, dz, Szz);
+      cnt += in;
+    };
     for (int cz = z0; cz <= z1; ++cz) {
       const float ez = fmaxf(0.f, fmaxf((float)cz - u[2], u[2] - (float)(cz + 1)));
       for (int cy = y0; cy <= y1; ++cy) {
@@ -297,32 +331,17 @@ __global__ void __launch_bounds__(128, 4) dpca_normal_kernel(const float4* __res
           const float bx = fmaxf(0.f, fmaxf(blo.x - q.x, q.x - bhi.x));
           const float by = fmaxf(0.f, fmaxf(blo.y - q.y, q.y - bhi.y));
           const float bz = fmaxf(0.f, fmaxf(blo.z - q.z, q.z - bhi.z));
-          const float b2 = __fadd_rn(__fadd_rn(__fmul_rn(bx, bx), __fmul_rn(by, by)), __fmul_rn(bz, bz));
-          if (!__any_sync(kFull, b2 <= r2)) continue;
+          if (!__any_sync(kFull, dist2_rn(bx, by, bz) <= r2)) continue;
           const int j0 = max(gs, s0), j1 = min(gs + kDpcaBox, s1);
-#pragma unroll 2
-          for (int j = j0 + ((sl - j0) & (kDpcaLanes - 1)); j < j1; j += kDpcaLanes) {
-            const float4 pj = sorted[j];
-            float dx = pj.x - q.x, dy = pj.y - q.y, dz = pj.z - q.z;
-            const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-            const bool in = d2 <= r2;
-            dx = in ? dx : 0.f;
-            dy = in ? dy : 0.f;
-            dz = in ? dz : 0.f;
-            const float w = in ? approx_rcp(fmaf(approx_sqrt(d2), inv_r, eps_r)) : 0.f;   // R w
-            const float wu = w * inv_r;
-            const float wx = wu * dx, wy = wu * dy, wz = wu * dz;   // R w y, y = (x_j - x_i) / R
-            S0 += w;
-            S1x += wx;
-            S1y += wy;
-            S1z += wz;
-            Sxx = fmaf(wx, dx, Sxx);   // R^2 w y y^T: one more 1/R below
-            Sxy = fmaf(wx, dy, Sxy);
-            Sxz = fmaf(wx, dz, Sxz);
-            Syy = fmaf(wy, dy, Syy);
-            Syz = fmaf(wy, dz, Syz);
-            Szz = fmaf(wz, dz, Szz);
-            cnt += in;
+          if (j1 - j0 == kDpcaBox) {   // whole: all of a lane's loads first
+            float4 pj[kDpcaBox / kDpcaLanes];
+#pragma unroll
+            for (int e = 0; e < kDpcaBox / kDpcaLanes; ++e) pj[e] = sorted[gs + sl + e * kDpcaLanes];
+#pragma unroll
+            for (int e = 0; e < kDpcaBox / kDpcaLanes; ++e) add(pj[e]);
+          } else {
+#pragma unroll 1
+            for (int j = j0 + ((sl - j0) & (kDpcaLanes - 1)); j < j1; j += kDpcaLanes) add(sorted[j]);
           }
         }
       }
