@@ -283,7 +283,8 @@ size_t dense_table_floats(int max_res) {
 
 // The tables for n, and the shared-memory opt-in of the pass kernels (kept out
 // of any capture of the handle's own).  Under the caller's capture the tables
-// are part of what is captured and count as not yet made.
+// are part of what is captured, and a replay may come between any two calls:
+// from then on every call makes its own (dense_n stays -1).
 int dense_setup(wgeo_handle* h, int n, cudaStream_t s) {
   if (!h->dense_attr) {
     const int most = (int)smem_bytes(kMaxRes);
@@ -292,15 +293,16 @@ int dense_setup(wgeo_handle* h, int n, cudaStream_t s) {
     WGEO_CUDA_TRY(cudaFuncSetAttribute(dense_pass_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     h->dense_attr = true;
   }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  WGEO_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) h->dense_n = -1;
   if (h->dense_n == n) return WGEO_OK;
   float* fwd = h->dense_tab;
   float* inv = fwd + (size_t)red_pad(n) * table_row(n);
   float* sk = inv + (size_t)red_pad(n) * table_row(n);
   dense_tables_kernel<<<grid_blocks((int64_t)red_pad(n) * table_row(n), 256), 256, 0, s>>>(n, fwd, inv, sk);
   WGEO_LAUNCH_CHECK();
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  WGEO_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
-  h->dense_n = cap == cudaStreamCaptureStatusNone ? n : 0;
+  if (h->dense_n >= 0) h->dense_n = n;
   return WGEO_OK;
 }
 

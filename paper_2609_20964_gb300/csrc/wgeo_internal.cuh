@@ -403,7 +403,7 @@ struct wgeo_handle {
   bool dct_attr = false;         // shared-memory opt-in of the pass kernels done (per device)
   // dense cosine transforms of the other grids: forward basis, inverse basis, eigenvalue factors
   float* dense_tab = nullptr;
-  int dense_n = 0;               // n the tables hold (0: none yet)
+  int dense_n = 0;               // n the tables hold (0: none yet, -1: made by every call)
   bool dense_attr = false;
 
   // points

@@ -67,3 +67,30 @@ def test_one_handle_over_several_grids(W):
         assert float((a - b).norm() / b.norm()) <= 1e-6
         one.close()
     rec.close()
+
+
+def test_a_captured_solve_leaves_other_grids_their_tables(W):
+    """The tables that a replay of one grid's backward writes are not taken for
+    those of the grid solved before it."""
+    p, n = synth.sphere_cloud(2000, seed=9)
+    rec = W(72, len(p))
+    P, N = _t(p), _t(n)
+    seed = {res: _t(np.random.default_rng(res).standard_normal((res, res, res)).astype(np.float32)) for res in (44, 72)}
+
+    def eager(res):
+        rec.reconstruct(P, N, BBOX, res)
+        return [x.clone() for x in rec.backward(d_sdf_grid=seed[res])[:2]]
+
+    want = {res: eager(res) for res in (72, 44)}
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got44 = rec.backward(d_sdf_grid=seed[44])[:2]
+    eager(72)
+    rec.reconstruct(P, N, BBOX, 44)
+    graph.replay()
+    for a, b in zip(got44, want[44]):
+        assert (a - b).norm() <= 1e-5 * b.norm()
+    for a, b in zip(eager(72), want[72]):
+        assert (a - b).norm() <= 1e-5 * b.norm()
+    rec.close()
