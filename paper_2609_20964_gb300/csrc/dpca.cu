@@ -232,7 +232,7 @@ __device__ __forceinline__ float jacobi_min_vector(float a[3][3], float v_out[3]
 // entry, none of them shared between points).  Groups that lie wholly in the
 // row's range, nearly all of them, run a lane's four entries unrolled with the
 // four loads first, the partial ones a plain loop: 2 10^5 points of a sphere at
-// R = 0.1 (about 4600 neighbours) 2831 -> 2390 us, 10^6 at 50 neighbours a disc
+// R = 0.1 (about 4100 neighbours) 2831 -> 2390 us, 10^6 at 50 neighbours a disc
 // 1130 -> 1020 (1060 without the bound of 8 blocks an SM on the registers).
 //
 // Weights.  w' = R w = 1 / (d / R + eps / R), at most R / eps <= 1e6, from the
