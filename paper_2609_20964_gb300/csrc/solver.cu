@@ -746,9 +746,15 @@ __global__ void __launch_bounds__(kSX * kSY) prolong_pair_kernel(const float* __
 // transforms give the same correction to FP32 rounding (chi unchanged to
 // ~1e-10 of its spread).  Forward solve at 120^3 (coarsest 15^3): 34.1 -> 1.0
 // ms; at 88^3 (11^3): 9.5 -> 0.8 ms.
+// A lone level that is the grid itself (its caller passes `shift`; coarse
+// levels have none) takes kPolish sweeps more: the transforms round every value
+// at the scale of the largest, which leaves 2 to 3 times the residual that
+// relaxation ends at (1.1e-6 of ||b|| at 15^3 against 3.7e-7), and the plain
+// FP32 mode, which has no refinement, then misses its 1e-6.
 constexpr int kSmallCap = 4096 + 512 + 64 + 27 + 8;
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallQ = 15 * 15;    // cosine basis of the largest coarsest level
+constexpr int kPolish = 8;          // sweeps after the direct solve of a whole grid (from 4 on the residual stays)
 
 // `sweeps` red-black sweeps, colour `first` first.  A thread owns up to two
 // pairs of x neighbours (one cell of each colour; found once, not per sweep)
@@ -915,6 +921,11 @@ __global__ void __launch_bounds__(kSmallThreads) small_vcycle_kernel(float* __re
     } else {
       small_basis(qs, n);
       small_direct(x, b, n, qs, false);
+      if (shift && L == 1) {   // the whole grid; the solve used b up
+        for (int t = threadIdx.x; t < N0; t += blockDim.x) bsm[t] = (bg[t] - sh) - meanb;
+        __syncthreads();
+        small_rbgs(x, b, n, kPolish, 0);
+      }
     }
   }
   // up
@@ -1042,6 +1053,11 @@ __global__ void __launch_bounds__(kSmallThreads) small_vcycle_q1_kernel(float* _
     } else {
       small_basis(qs, n);
       small_direct(x, b, n, qs, true);
+      if (shift && L == 1) {   // the whole grid; the solve used b up
+        for (int t = threadIdx.x; t < N0; t += blockDim.x) bsm[t] = (bg[t] - sh) - meanb;
+        __syncthreads();
+        small_gs8(x, b, n, kPolish, 0, 1);
+      }
     }
   }
   for (int l = L - 2; l >= 0; --l) {

@@ -42,3 +42,22 @@ def test_forward_solve_matches_the_oracle(W, res, galerkin):
     # a relaxed solve stops at 1e-6 of ||b||; the bound of the parity tests
     assert np.abs((chi - chi.mean()) - (ref.chi - ref.chi.mean())).max() <= 1e-4 * span
     rec.close()
+
+
+@pytest.mark.parametrize("cloud", ["sphere", "sheet"])
+@pytest.mark.parametrize("res", [4, 5, 7, 9, 11, 13, 15])
+def test_a_lone_level_is_solved_to_float32_rounding(W, res, cloud):
+    """The plain FP32 mode has no refinement: on a grid that is one level the
+    one solve has to reach the tolerance by itself."""
+    from paper_2609_20964_gb300 import PREC_FP32
+    p, n = synth.sphere_cloud(4000, seed=res)
+    if cloud == "sheet":
+        p = np.random.default_rng(res).uniform(0.1, 0.9, p.shape).astype(np.float32)
+        p[:, 2] = 0.5
+        n = np.tile(np.float32([0, 0, 1]), (len(p), 1))
+    rec = W(res, len(p), precision=PREC_FP32)
+    rec.reconstruct(_t(p), _t(n), BBOX, res)
+    info = rec.info()
+    assert info["status"] == 0 and info["solver_steps"] == 1, info
+    assert info["residual_rel"] <= 1e-6, info
+    rec.close()
