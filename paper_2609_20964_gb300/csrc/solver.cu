@@ -1878,13 +1878,14 @@ int spectral_setup(wgeo_handle* h, int n, cudaStream_t s) {
     WGEO_CUDA_TRY(dct_attr<16>());
     h->dct_attr = true;
   }
-  if (h->dct_n != n) {
-    dct_tables_kernel<<<div_up(n > 160 ? n + 1 : 161, 256), 256, 0, s>>>(n, h->dct_t1, h->dct_w32, h->dct_wml,
-                                                                         h->dct_tr, h->dct_sk, h->dct_skl,
-                                                                         h->dct_tw, h->dct_wq);
-    WGEO_LAUNCH_CHECK();
-    h->dct_n = n;
-  }
+  int rc = tables_for_capture(h->dct_n, s);
+  if (rc) return rc;
+  if (h->dct_n == n) return WGEO_OK;
+  dct_tables_kernel<<<div_up(n > 160 ? n + 1 : 161, 256), 256, 0, s>>>(n, h->dct_t1, h->dct_w32, h->dct_wml,
+                                                                       h->dct_tr, h->dct_sk, h->dct_skl,
+                                                                       h->dct_tw, h->dct_wq);
+  WGEO_LAUNCH_CHECK();
+  if (h->dct_n >= 0) h->dct_n = n;
   return WGEO_OK;
 }
 

@@ -281,10 +281,19 @@ size_t dense_table_floats(int max_res) {
   return 2 * (size_t)red_pad(max_res) * table_row(max_res) + (size_t)max_res;
 }
 
+// Under the caller's capture a solve's tables are part of what is captured, and
+// a replay may come between any two calls, on another grid than the last one's:
+// from then on every call of the handle makes its own (`held`, the grid that the
+// tables are known to hold, stays -1).
+int tables_for_capture(int& held, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  WGEO_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) held = -1;
+  return WGEO_OK;
+}
+
 // The tables for n, and the shared-memory opt-in of the pass kernels (kept out
-// of any capture of the handle's own).  Under the caller's capture the tables
-// are part of what is captured, and a replay may come between any two calls:
-// from then on every call makes its own (dense_n stays -1).
+// of any capture of the handle's own).
 int dense_setup(wgeo_handle* h, int n, cudaStream_t s) {
   if (!h->dense_attr) {
     const int most = (int)smem_bytes(kMaxRes);
@@ -293,9 +302,8 @@ int dense_setup(wgeo_handle* h, int n, cudaStream_t s) {
     WGEO_CUDA_TRY(cudaFuncSetAttribute(dense_pass_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     h->dense_attr = true;
   }
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  WGEO_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
-  if (cap != cudaStreamCaptureStatusNone) h->dense_n = -1;
+  int rc = tables_for_capture(h->dense_n, s);
+  if (rc) return rc;
   if (h->dense_n == n) return WGEO_OK;
   float* fwd = h->dense_tab;
   float* inv = fwd + (size_t)red_pad(n) * table_row(n);

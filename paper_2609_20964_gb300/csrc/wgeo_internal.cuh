@@ -399,7 +399,7 @@ struct wgeo_handle {
   float2* dct_wq = nullptr;      //   e^{-i pi q / (2 n)} (q <= n)
   float* dct_sk = nullptr;       //   4 sin^2(pi k / (2 n)) (k < n, natural order)
   float* dct_skl = nullptr;      //   the same at k = a + R brev5(j)
-  int dct_n = 0;                 // n the tables hold (0: none yet)
+  int dct_n = 0;                 // n the tables hold (0: none yet, -1: made by every call)
   bool dct_attr = false;         // shared-memory opt-in of the pass kernels done (per device)
   // dense cosine transforms of the other grids: forward basis, inverse basis, eigenvalue factors
   float* dense_tab = nullptr;
@@ -541,6 +541,7 @@ int launch_unpack_bins(wgeo_handle* h, int* out, cudaStream_t s);
 int launch_solve(wgeo_handle* h, int res, int mode, bool cold, cudaStream_t s);
 // spectral_dense.cu: the direct correction on grids without an FFT pass
 size_t dense_table_floats(int max_res);
+int tables_for_capture(int& held, cudaStream_t s);   // dct_n, dense_n
 int dense_setup(wgeo_handle* h, int n, cudaStream_t s);
 int dense_solve(wgeo_handle* h, int n, float* e, const float* r, const int* gate, cudaStream_t s);
 // surface.cu

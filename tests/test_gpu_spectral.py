@@ -134,3 +134,33 @@ def test_spectral_adjoint_at_256_agrees_with_multigrid(W, galerkin):
     (a, sa), (b, sb) = out
     assert np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(b)
     assert sa <= 4 and sa <= sb
+
+
+def test_a_captured_step_and_eager_ones_keep_their_own_tables(W):
+    """A captured forward and backward writes the cosine tables of its grid at
+    every replay, and an eager call after one does not take them for its own."""
+    p, n = synth.sphere_cloud(3000, seed=11)
+    P, N = _t(p), _t(n)
+    seed = {res: _t(np.random.default_rng(res).standard_normal((res, res, res)).astype(np.float32)) for res in (64, 128)}
+    rec = W(128, len(p))
+
+    def step(res):
+        sdf, _ = rec.reconstruct(P, N, BBOX, res)
+        return (sdf, *rec.backward(d_sdf_grid=seed[res])[:2])
+
+    def close(got, want):
+        # repeats differ by the order of the atomics
+        return all(bool((a - b).norm() <= 1e-5 * b.norm()) for a, b in zip(got, want))
+
+    want = {res: [x.clone() for x in step(res)] for res in (128, 64)}
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = step(64)
+    assert close(step(128), want[128])
+    graph.replay()
+    torch.cuda.synchronize()
+    assert close(got, want[64])
+    assert close(step(128), want[128])
+    assert rec.info()["status"] == 0
+    rec.close()
