@@ -2026,14 +2026,21 @@ __global__ void __launch_bounds__(kPatchWarps * 32, 4) sdf_patch_kernel(const __
 // chi >= c (c double) is tested as chi >= the smallest float not below c, so no
 // node needs FP64.
 //
-// Candidates of one class (the top 32 - id_bits bits of feature_class; id_bits
-// 0: none) are not told apart here: the float32 distance, and where that is
-// equal the order of the candidate list, decides between them beforehand.  The nodes' results
-// have always been those of this rule (one pair of features in 2^(32 -
-// id_bits)), and a node between two triangles whose vertices are sensitive can
-// carry 5e-5 of a dense gradient's norm to one or the other.  The
-// seeds are the triangles of the stride-2 lattice around the node.  The nodes of that lattice (even != 0) take their
-// own pass, after the others have read their triangles.
+// Candidates of one class (the top 32 - id_bits bits of feature_class) are not
+// told apart here: the float32 distance, and where that is equal the order of
+// the candidate list, decides between them beforehand.  Candidates that share
+// their closest vertex or edge are of one class and the same closest point;
+// distinct features meet in one by chance, two vertices about once in 1000
+// (their ten bits), others once in 2^(32 - id_bits).  At such a node (50 of 16.8
+// million at 256^3) the float32 choice stands, right to 4e-7 of the distance but
+// not always the nearer one.  Deciding those in float-float too lowers the
+// error of a dense 120^3 gradient against 64 bits by 0.2 to 8% (3.92e-4 -> 3.91e-4,
+// 1.73e-6 -> 1.60e-6) but moves gradients of 256^3 grids by up to 4e-5 of their
+// norm, past the 1e-5 that results are kept to from version to version: the
+// rule stays.  id_bits comes from the grid, so that the choice does not depend on
+// the handle's capacities.  The seeds are the triangles of the stride-2 lattice
+// around the node.  The nodes of that lattice (even != 0) take their own pass,
+// after the others have read their triangles.
 __global__ void sdf_tie_kernel(const __grid_constant__ Search S, SurfParams g, int id_bits, int even) {
   __shared__ float2 s_ax[3][kMaxRes];
   const int n = g.res;
@@ -2058,28 +2065,26 @@ __global__ void sdf_tie_kernel(const __grid_constant__ Search S, SurfParams g, i
     const float2 px = s_ax[0][i], py = s_ax[1][j], pz = s_ax[2][k];
     const float3 p = make_float3(px.x, py.x, pz.x);
     int left = 0;
-    if (id_bits > 0) {
-      float d2[kCand];
-      unsigned cls[kCand];
+    float d2[kCand];
+    unsigned cls[kCand];
 #pragma unroll 1
-      for (int q = 0; q < kCand; ++q) {
-        if (cand[q] < 0) continue;
-        float v, w;
-        d2[q] = tri_dist2_rec(p, S.tris_s + kTriRec * (int64_t)cand[q], v, w);
-        cls[q] = feature_class(v, w, S.tris, cand[q]) >> id_bits;
-        for (int r = 0; r < q && cand[q] >= 0; ++r) {
-          if (cand[r] < 0 || cls[r] != cls[q]) continue;
-          bool stays = d2[r] < d2[q];
-          if (d2[r] == d2[q]) {
-            int seeds[8];
-            for (int c = 0; c < 8; ++c) {
-              const int ci = (i & ~1) + 2 * (c & 1), cj = (j & ~1) + 2 * ((c >> 1) & 1), ck = (k & ~1) + 2 * (c >> 2);
-              seeds[c] = !even && ci < n && cj < n && ck < n ? S.ctri[lin3(ci, cj, ck, n)] : -1;
-            }
-            stays = comes_first(cand[r], cand[q], S.tris_lo, seeds);
+    for (int q = 0; q < kCand; ++q) {
+      if (cand[q] < 0) continue;
+      float v, w;
+      d2[q] = tri_dist2_rec(p, S.tris_s + kTriRec * (int64_t)cand[q], v, w);
+      cls[q] = feature_class(v, w, S.tris, cand[q]) >> id_bits;
+      for (int r = 0; r < q && cand[q] >= 0; ++r) {
+        if (cand[r] < 0 || cls[r] != cls[q]) continue;
+        bool stays = d2[r] < d2[q];
+        if (d2[r] == d2[q]) {
+          int seeds[8];
+          for (int c = 0; c < 8; ++c) {
+            const int ci = (i & ~1) + 2 * (c & 1), cj = (j & ~1) + 2 * ((c >> 1) & 1), ck = (k & ~1) + 2 * (c >> 2);
+            seeds[c] = !even && ci < n && cj < n && ck < n ? S.ctri[lin3(ci, cj, ck, n)] : -1;
           }
-          cand[stays ? q : r] = -1;
+          stays = comes_first(cand[r], cand[q], S.tris_lo, seeds);
         }
+        cand[stays ? q : r] = -1;
       }
     }
 #pragma unroll
@@ -2723,10 +2728,10 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
   stage_end(h, kStSDF, slot, s);
   if (ctri) {
     slot = stage_begin(h, kStSDFTie, s);
-    // bits of a triangle id (ids < cap <= 2^id_bits - 1; at most 24)
-    int id_bits = 0;
-    while (id_bits < 32 && ((int64_t)1 << id_bits) - 1 < h->mesh_cap) ++id_bits;
-    if (id_bits > 24) id_bits = 0;
+    // bits of a triangle id under the default capacity of this grid (at least
+    // 4096 triangles; at most 24 bits, 16 * 800^2)
+    int id_bits = 13;
+    while (((int64_t)1 << id_bits) - 1 < (int64_t)16 * res * res) ++id_bits;
     sdf_tie_kernel<<<152 * 8, 256, 0, s>>>(S, g, id_bits, 0);
     WGEO_LAUNCH_CHECK();
     sdf_tie_kernel<<<152 * 8, 256, 0, s>>>(S, g, id_bits, 1);

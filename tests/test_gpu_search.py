@@ -79,3 +79,18 @@ def test_search_in_a_box_far_from_the_origin(W):
     sdf, _ = rec.reconstruct(_t(p + off), _t(n), bbox, res, with_normals=False)
     _check(rec, sdf, res, bbox, np.random.default_rng(0).choice(res ** 3, 3000, replace=False))
     rec.close()
+
+
+def test_closest_triangles_do_not_depend_on_the_capacities(W):
+    """The mesh capacity and the largest grid of a handle only size its
+    buffers: near-ties go the same way under any of them."""
+    res, bbox = 128, np.array([0, 0, 0, 1, 1, 1], dtype=np.float32)
+    p, n, _ = synth.sh_body_cloud(60_000, seed=res)
+    want = None
+    for max_res, cap in ((res, 0), (res, 100 * res * res), (res, 15_000_000), (res, 17_000_000), (2 * res, 0)):
+        rec = W(max_res, len(p), mesh_capacity=cap)
+        rec.reconstruct(_t(p), _t(n), bbox, res)
+        got = [rec.field(name).clone() for name in ("closest", "phi")]
+        rec.close()
+        want = want or got
+        assert all(torch.equal(a, b) for a, b in zip(got, want)), (max_res, cap)
