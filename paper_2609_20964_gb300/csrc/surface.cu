@@ -1346,13 +1346,16 @@ __device__ __forceinline__ float reach_of(const float3 p0, const float3 y, float
   return u + 2.f * m * (1e-6f * m + 5e-7f * coord);
 }
 
-// Squared distance from p to a triangle without branches, to rank triangles:
+// Squared distance d^2 from p to a triangle without branches, to rank triangles:
 // the least of the three clamped edges and, when the projection falls inside,
 // the face, each as a quadratic form about vertex a (stationary in the
-// weights, so their rounding enters to second order).  Its error is below 1e-6
-// (|p - a|^2), a cancellation that tri_dist2_rec avoids; |p - a|^2 exceeds the
-// squared distance by at most the squared longest edge (3 h^2) where the
-// closest point lies on the triangle.
+// weights, so their rounding enters to second order).  Its error is the
+// cancellation against |p - a|^2, which tri_dist2_rec avoids, below 1e-6 (d +
+// sqrt(3) h)^2 (edges are at most the cube's diagonal; 4e-7 (d^2 + 3 h^2)
+// measured), and on thin triangles that of the face weights: they are off by
+// about the rounding times (edge / height)^2, and the smaller of the face at
+// such weights and the edges exceeds d^2 by up to 4.0e-5 h^2 (worst of 6e7
+// triangles tried, at a height of 0.007 edges).
 __device__ __forceinline__ float tri_dist2_fast(const float3 p, const float4* __restrict__ rec) {
   const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
   const float3 ap = make_float3(p.x - r0.x, p.y - r0.y, p.z - r0.z);
@@ -1373,11 +1376,16 @@ __device__ __forceinline__ float tri_dist2_fast(const float3 p, const float4* __
   return fmaxf(in ? fminf(q, qf) : q, 0.f);
 }
 
-// The cut that goes with a distance of tri_dist2_fast: margin2 widened by its
-// error (the square root by the hardware's approximation, from above).
+// The cut that goes with a distance of tri_dist2_fast: the near-tie margin
+// (Cands::reach) widened by the errors of this distance and of the one to be
+// admitted, 2e-6 (d + sqrt(3) h)^2 <= 3e-6 d^2 + 1.8e-5 h^2 of cancellation and
+// 4e-5 h^2 of thin triangles (the square root by the hardware's approximation,
+// from above).
+constexpr float kFastRel = 4e-6f;   // of d^2, 8e-7 of it the near-tie margin's
+constexpr float kFastAbs = 1e-4f;   // of h^2
 __device__ __forceinline__ float fast_cut(float q, float mabs, float h2) {
   const float m = 2.f * mabs;
-  return fmaf(q, 1.f + 4e-6f, fmaf(2.001f * m, q * rsqrtf(fmaxf(q, 1e-30f)), fmaf(m, m, 1e-5f * h2)));
+  return fmaf(q, 1.f + kFastRel, fmaf(2.001f * m, q * rsqrtf(fmaxf(q, 1e-30f)), fmaf(m, m, kFastAbs * h2)));
 }
 
 // Closest point to p on triangle t (its search record).
