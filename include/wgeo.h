@@ -99,7 +99,8 @@ typedef struct {
                                 takes each refinement step's correction from a direct spectral
                                 solve (the operator is diagonal in the cosine basis of the mirrored
                                 walls; always two steps), and FP32 mode solves once, directly; on
-                                every other res the adjoint solve does so, in two steps as well;
+                                every other res up to 512 (with galerkin: on every other res) the
+                                adjoint solve does so, in two steps as well;
                                 0: multigrid V-cycles on every grid */
   int32_t reserved[3];
   double  tol_rel_adjoint;   /* adjoint solve: stop when ||g - A lambda|| <= tol * ||g|| (default 1e-7) */

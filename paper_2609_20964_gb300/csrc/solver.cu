@@ -1202,11 +1202,12 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // Whether the FFT passes take this grid, and whether a solve's correction is a
 // direct spectral one: on the other grids the dense transforms
-// (spectral_dense.cu) give it to the adjoint solve, while forward solves keep
-// their V-cycles (and with them chi, warm starts and the plain FP32 mode).
+// (spectral_dense.cu) give it to the adjoint solve up to dense_limit, while
+// forward solves keep their V-cycles (and with them chi, warm starts and the
+// plain FP32 mode).
 bool fft_grid(int n) { return n >= 32 && n <= 512 && (n & (n - 1)) == 0; }
 bool use_spectral(const wgeo_handle* h, int n, int mode) {
-  return h->opt.spectral && (fft_grid(n) || mode == 1);
+  return h->opt.spectral && (fft_grid(n) || (mode == 1 && n <= dense_limit(h->opt.galerkin)));
 }
 
 __host__ __device__ constexpr int dct_ls(int n) { return (n + n / 32) | 1; }   // odd row stride

@@ -1,5 +1,5 @@
 // Spectral correction of the adjoint solve on grids that the FFT passes do not
-// take (n not a power of two, or below 32): the same direct solve of L e = r -
+// take (n not a power of two, or below 32), up to dense_limit: the same direct solve of L e = r -
 // mean(r) in the cosine basis (solver.cu), each one-dimensional transform as a
 // dense product folded by the basis' symmetry.  The forward solves of these
 // grids stay with their V-cycles: chi decides which of two nearly equidistant
@@ -20,7 +20,9 @@
 // product of this size is a few tens of microseconds at the FP32 rate of this
 // GPU.  Bound: FP32 issue, 32 FMA per 4 shared 16-byte loads.  Adjoint solve
 // (two corrections and residuals) against the V-cycles, ms: 0.20 / 0.80 at
-// 88^3, 0.30 / 1.8 (unlumped operator) at 96^3, 0.30 / 1.0 at 120^3.
+// 88^3, 0.30 / 1.8 (unlumped operator) at 96^3, 0.30 / 1.0 at 120^3; where the
+// n^4 operations catch up with the V-cycles' n^3 is dense_limit.  Line numbers
+// (n^2 of them) fit 32 bits, element offsets are 64-bit.
 #include "wgeo_internal.cuh"
 
 namespace wgeo {

@@ -541,6 +541,13 @@ int launch_unpack_bins(wgeo_handle* h, int* out, cudaStream_t s);
 int launch_solve(wgeo_handle* h, int res, int mode, bool cold, cudaStream_t s);
 // spectral_dense.cu: the direct correction on grids without an FFT pass
 size_t dense_table_floats(int max_res);
+// The largest such grid: the transforms' n^4 operations meet the V-cycles' n^3
+// between 480^3 and 576^3 for the lumped operator (adjoint solve, dense /
+// V-cycles, ms: 448^3 17.3 / 23.2, 480^3 27.6 / 31.2, 576^3 53.2 / 50.5, 640^3
+// 72.8 / 67.4, 768^3 141 / 113).  The unlumped one's V-cycles cost twice as
+// much and stay behind up to the largest grid (480^3 35.2 / 55.9, 640^3 89.9 /
+// 127.7, 768^3 171 / 220).
+inline int dense_limit(int galerkin) { return galerkin ? kMaxRes : 512; }
 int tables_for_capture(int& held, cudaStream_t s);   // dct_n, dense_n
 int dense_setup(wgeo_handle* h, int n, cudaStream_t s);
 int dense_solve(wgeo_handle* h, int n, float* e, const float* r, const int* gate, cudaStream_t s);

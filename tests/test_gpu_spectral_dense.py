@@ -94,3 +94,21 @@ def test_a_captured_solve_leaves_other_grids_their_tables(W):
     for a, b in zip(eager(72), want[72]):
         assert (a - b).norm() <= 1e-5 * b.norm()
     rec.close()
+
+
+@pytest.mark.parametrize("res, galerkin, direct", [(320, 0, True), (576, 0, False), (576, 1, True)])
+def test_adjoint_of_large_grids_against_the_v_cycles(W, res, galerkin, direct):
+    """Direct up to the line where the V-cycles are faster; both ways the
+    gradient is that of a handle without spectral solves."""
+    p, n = synth.sphere_cloud(20_000, seed=5)
+    g = torch.randn((res, res, res), device="cuda", generator=torch.Generator("cuda").manual_seed(res))
+    out = []
+    for spectral in (1, 0):
+        rec = W(res, len(p), galerkin=galerkin, spectral=spectral)
+        rec.reconstruct(_t(p), _t(n), BBOX, res, with_normals=False)
+        out.append(rec.backward(d_sdf_grid=g)[0])
+        steps = rec.info()["backward_steps"]
+        assert (steps == 2) == (direct and spectral == 1), steps
+        rec.close()
+    # the V-cycles stop at 1e-7 of the right-hand side
+    assert float((out[0] - out[1]).norm() / out[1].norm()) <= 1e-6
