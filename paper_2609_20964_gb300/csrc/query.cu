@@ -122,94 +122,179 @@ __global__ void query_kernel(const float* __restrict__ q, int64_t m, QParams g,
   }
 }
 
-// phi and the normal: four lanes per query.  The gradients at the cell's eight
+// phi and the normal of a query: the terms of the cell's corners, each operation
+// rounded as written, so that the two forms below give the same bits and a
+// result does not depend on the other queries of the call.
+struct NormalSum {
+  float s = 0.f, mv[3] = {0.f, 0.f, 0.f};
+  // a corner of weight w, value c and differences d (times 2 h)
+  __device__ __forceinline__ void add(float w, float c, float dx, float dy, float dz, float inv2h) {
+    const float gr[3] = {__fmul_rn(dx, inv2h), __fmul_rn(dy, inv2h), __fmul_rn(dz, inv2h)};
+    const float m2 = __fmaf_rn(gr[2], gr[2], __fmaf_rn(gr[1], gr[1], __fmul_rn(gr[0], gr[0])));
+    const float inv = (isfinite(m2) && m2 > 0.f) ? rsqrtf(m2) : 0.f;
+    s = __fmaf_rn(w, c, s);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) mv[a] = __fmaf_rn(__fmul_rn(w, gr[a]), inv, mv[a]);
+  }
+  // 1 / |mv|, 0 for no direction
+  __device__ __forceinline__ float inv_norm() const {
+    const float m2 = __fmaf_rn(mv[2], mv[2], __fmaf_rn(mv[1], mv[1], __fmul_rn(mv[0], mv[0])));
+    return (m2 > 0.f) ? rsqrtf(m2) : 0.f;
+  }
+};
+
+// Difference at the lower (up = 0) or upper node of v1, v2 in the window v,
+// one-sided on the grid's first and last node.
+__device__ __forceinline__ float node_diff(bool up, bool fst, bool lst, float v0, float v1, float v2, float v3) {
+  if (up) return lst ? __fmaf_rn(3.f, v2, __fmaf_rn(-4.f, v1, v0)) : __fsub_rn(v3, v1);
+  return fst ? __fmaf_rn(-3.f, v1, __fmaf_rn(4.f, v2, -v3)) : __fsub_rn(v2, v0);
+}
+
+__device__ __forceinline__ float corner_weight(float fx, const float t[3], int by, int bz) {
+  return __fmul_rn(__fmul_rn(fx, by ? t[1] : 1.f - t[1]), bz ? t[2] : 1.f - t[2]);
+}
+
+// phi and the normal, four lanes per query.  The gradients at the cell's eight
 // corners take the 4 x 4 x 4 nodes around it less its edges and corners (32
 // values); lane l of a query reads the columns at x = i0 - 1 + l, so one load
-// instruction touches the rows of eight queries instead of one line per lane
-// (the L1 takes a line at a time: 56 gathers a thread were its bound, 131 us for
-// 1M queries at 128^3; twelve loads now, 74 us, bound by issue: 59 instructions a
-// query, 65% of the slots).  Lanes 1 and 2 hold the
-// corners: y and z differences are their own, x differences come from the
-// neighbouring lanes.  A cell at the grid's edge uses the one-sided stencils on
-// the same window (its clamped columns are not used).
+// instruction touches the rows of eight queries instead of one line per lane.
+// Lanes 1 and 2 hold the corners: y and z differences are their own, x
+// differences come from the neighbouring lanes.  A cell at the grid's edge uses
+// the one-sided stencils on the same window (its clamped columns are not used).
+// Lanes 0 to 2 write the normal, lane 3 the distance.
+__device__ __forceinline__ void query_normal_lanes(const int i0[3], const float t[3], int64_t i, bool on, int n,
+                                                   float inv2h, const float* __restrict__ phi,
+                                                   float* __restrict__ sdf_q, float* __restrict__ nrm_q) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int nn = n * n;
+  const int lane = threadIdx.x & 31, l = lane & 3;
+  const bool corner = l == 1 || l == 2;
+  const bool first[3] = {i0[0] == 0, i0[1] == 0, i0[2] == 0};
+  const bool last[3] = {i0[0] == n - 2, i0[1] == n - 2, i0[2] == n - 2};
+  const float* col = phi + min(max(i0[0] - 1 + l, 0), n - 1);
+  const int y1 = i0[1] * n, z1 = i0[2] * nn, y2 = y1 + n, z2 = z1 + nn;
+  // centre columns (y + 2 z), and the y and z neighbours of the corner lanes
+  const float c[4] = {col[y1 + z1], col[y2 + z1], col[y1 + z2], col[y2 + z2]};
+  float ya[2] = {0.f, 0.f}, yb[2] = {0.f, 0.f}, za[2] = {0.f, 0.f}, zb[2] = {0.f, 0.f};
+  if (corner) {
+    const int y0 = first[1] ? y1 : y1 - n, y3 = last[1] ? y2 : y2 + n;
+    const int z0 = first[2] ? z1 : z1 - nn, z3 = last[2] ? z2 : z2 + nn;
+    ya[0] = col[y0 + z1], ya[1] = col[y0 + z2], yb[0] = col[y3 + z1], yb[1] = col[y3 + z2];
+    za[0] = col[y1 + z0], za[1] = col[y2 + z0], zb[0] = col[y1 + z3], zb[1] = col[y2 + z3];
+  }
+  const float fx = l == 2 ? t[0] : 1.f - t[0];
+  NormalSum a;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int by = k & 1, bz = k >> 1;
+    const float prev = __shfl_sync(kFull, c[k], lane - 1), next = __shfl_sync(kFull, c[k], lane + 1),
+                far = __shfl_sync(kFull, c[k], lane ^ 2);
+    const float dx = l == 1 ? node_diff(false, first[0], false, prev, c[k], next, far)
+                            : node_diff(true, false, last[0], far, prev, c[k], next);
+    const float dy = node_diff(by, first[1], last[1], ya[bz], c[2 * bz], c[2 * bz + 1], yb[bz]);
+    const float dz = node_diff(bz, first[2], last[2], za[by], c[by], c[2 + by], zb[by]);
+    a.add(corner_weight(fx, t, by, bz), c[k], dx, dy, dz, inv2h);
+  }
+  // lanes 1 and 2 together
+  a.s += __shfl_xor_sync(kFull, a.s, 3);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) a.mv[k] += __shfl_xor_sync(kFull, a.mv[k], 3);
+  const float inv = a.inv_norm();
+  const int src = (lane & ~3) + 1;
+  const float o0 = __shfl_sync(kFull, a.mv[0] * inv, src), o1 = __shfl_sync(kFull, a.mv[1] * inv, src),
+              o2 = __shfl_sync(kFull, a.mv[2] * inv, src), o3 = __shfl_sync(kFull, a.s, src);
+  if (on) {
+    if (l == 3)
+      sdf_q[i] = o3;
+    else
+      nrm_q[3 * i + l] = l == 0 ? o0 : l == 1 ? o1 : o2;
+  }
+}
+
+// The same by one thread.
+__device__ __forceinline__ void query_normal_thread(const int i0[3], const float t[3], int64_t i, int n, float inv2h,
+                                                    const float* __restrict__ phi, float* __restrict__ sdf_q,
+                                                    float* __restrict__ nrm_q) {
+  const int nn = n * n;
+  const bool first[3] = {i0[0] == 0, i0[1] == 0, i0[2] == 0};
+  const bool last[3] = {i0[0] == n - 2, i0[1] == n - 2, i0[2] == n - 2};
+  const float* p = phi + ((i0[2] * n + i0[1]) * n + i0[0]);
+  const int xa = first[0] ? 0 : -1, xb = last[0] ? 1 : 2, y0 = first[1] ? 0 : -n, y3 = last[1] ? n : 2 * n,
+            z0 = first[2] ? 0 : -nn, z3 = last[2] ? nn : 2 * nn;
+  NormalSum a[2];   // by the corner's x
+  float c[4][4], ya[2][2], yb[2][2], za[2][2], zb[2][2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float* r = p + (k & 1) * n + (k >> 1) * nn;
+    c[k][0] = r[xa], c[k][1] = r[0], c[k][2] = r[1], c[k][3] = r[xb];
+  }
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      ya[x][b] = p[x + b * nn + y0], yb[x][b] = p[x + b * nn + y3];
+      za[x][b] = p[x + b * n + z0], zb[x][b] = p[x + b * n + z3];
+    }
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int by = k & 1, bz = k >> 1;
+      const float dx = node_diff(x, first[0], last[0], c[k][0], c[k][1], c[k][2], c[k][3]);
+      const float dy = node_diff(by, first[1], last[1], ya[x][bz], c[2 * bz][1 + x], c[2 * bz + 1][1 + x], yb[x][bz]);
+      const float dz = node_diff(bz, first[2], last[2], za[x][by], c[by][1 + x], c[2 + by][1 + x], zb[x][by]);
+      a[x].add(corner_weight(x ? t[0] : 1.f - t[0], t, by, bz), c[k][1 + x], dx, dy, dz, inv2h);
+    }
+  a[0].s += a[1].s;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) a[0].mv[k] += a[1].mv[k];
+  const float inv = a[0].inv_norm();
+  sdf_q[i] = a[0].s;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) nrm_q[3 * i + k] = a[0].mv[k] * inv;
+}
+
+// A warp takes 32 queries, a lane finding the cell of one.  What bounds it is the
+// L1, which serves one 128-byte line at a time: where no two of the warp's cells
+// lie on one line (scattered queries), four lanes a query touch a third of the
+// lines (1M at 128^3 88 us, 100 by one thread a query; 4M at 512^3 893 / 1285);
+// where two do (a lattice, rows, blocks of up to 32^3 cells), one thread a query
+// spends a third of the instructions (4M at 128^3, us: lattice 101, four lanes
+// 244; rows 106 / 245; blocks of 16^3 180 / 256, of 32^3, where half of the warps
+// share a line, 268 / 260).
 __global__ void __launch_bounds__(256) query_normal_kernel(const float* __restrict__ q, int64_t m, QParams g,
                                                            const float* __restrict__ phi, float* __restrict__ sdf_q,
                                                            float* __restrict__ nrm_q) {
   constexpr unsigned kFull = 0xffffffffu;
-  const int n = g.res, nn = n * n;
+  const int n = g.res;
   const float inv2h = (float)(0.5 / g.h);
-  const int lane = threadIdx.x & 31, l = lane & 3;
-  const bool corner = l == 1 || l == 2;
+  const int lane = threadIdx.x & 31;
   // warp-uniform trip count: every lane reaches the shuffles
-  for (int64_t base = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane) / 4; base < m;
-       base += (int64_t)gridDim.x * blockDim.x / 4) {
-    const int64_t i = min(base + (lane >> 2), m - 1);
-    // lane a finds the cell along axis a
-    const int ax = min(l, 2);
-    const float loh = ax == 0 ? g.lo_hi[0] : ax == 1 ? g.lo_hi[1] : g.lo_hi[2];
-    const float lol = ax == 0 ? g.lo_lo[0] : ax == 1 ? g.lo_lo[1] : g.lo_lo[2];
-    int my_i;
-    float my_t;
-    node_cell_ff(node_coord_ff(q[3 * i + ax], loh, lol, g.ih_hi, g.ih_lo), n, my_i, my_t);
-    int i0[3];
-    float t[3];
+  for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < m;
+       base += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t own = min(base + lane, m - 1);
+    int my_i[3];
+    float my_t[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      i0[a] = __shfl_sync(kFull, my_i, (lane & ~3) + a);
-      t[a] = __shfl_sync(kFull, my_t, (lane & ~3) + a);
+    for (int a = 0; a < 3; ++a)
+      node_cell_ff(node_coord_ff(q[3 * own + a], g.lo_hi[a], g.lo_lo[a], g.ih_hi, g.ih_lo), n, my_i[a], my_t[a]);
+    const unsigned same = __match_any_sync(kFull, ((my_i[2] * n + my_i[1]) * n + my_i[0]) >> 5);
+    if (__any_sync(kFull, (same & (same - 1u)) != 0u)) {
+      if (base + lane < m) query_normal_thread(my_i, my_t, own, n, inv2h, phi, sdf_q, nrm_q);
+      __syncwarp();
+      continue;
     }
-    const bool first[3] = {i0[0] == 0, i0[1] == 0, i0[2] == 0};
-    const bool last[3] = {i0[0] == n - 2, i0[1] == n - 2, i0[2] == n - 2};
-    const float* col = phi + min(max(i0[0] - 1 + l, 0), n - 1);
-    const int y1 = i0[1] * n, z1 = i0[2] * nn, y2 = y1 + n, z2 = z1 + nn;
-    // centre columns (y + 2 z), and the y and z neighbours of the corner lanes
-    const float c[4] = {col[y1 + z1], col[y2 + z1], col[y1 + z2], col[y2 + z2]};
-    float ya[2] = {0.f, 0.f}, yb[2] = {0.f, 0.f}, za[2] = {0.f, 0.f}, zb[2] = {0.f, 0.f};
-    if (corner) {
-      const int y0 = first[1] ? y1 : y1 - n, y3 = last[1] ? y2 : y2 + n;
-      const int z0 = first[2] ? z1 : z1 - nn, z3 = last[2] ? z2 : z2 + nn;
-      ya[0] = col[y0 + z1], ya[1] = col[y0 + z2], yb[0] = col[y3 + z1], yb[1] = col[y3 + z2];
-      za[0] = col[y1 + z0], za[1] = col[y2 + z0], zb[0] = col[y1 + z3], zb[1] = col[y2 + z3];
-    }
-    // difference at the lower (up = 0) or upper node of v[1], v[2] in the window v
-    auto diff = [](bool up, bool fst, bool lst, float v0, float v1, float v2, float v3) {
-      if (up) return lst ? 3.f * v2 - 4.f * v1 + v0 : v3 - v1;
-      return fst ? -3.f * v1 + 4.f * v2 - v3 : v2 - v0;
-    };
-    const float fx = l == 2 ? t[0] : 1.f - t[0];
-    float s = 0.f, mv[3] = {0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int r = 0; r < 32; r += 8) {
+      const int from = r + (lane >> 2);
+      int i0[3];
+      float t[3];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int by = k & 1, bz = k >> 1;
-      const float prev = __shfl_sync(kFull, c[k], lane - 1), next = __shfl_sync(kFull, c[k], lane + 1),
-                  far = __shfl_sync(kFull, c[k], lane ^ 2);
-      const float gx = l == 1 ? diff(false, first[0], false, prev, c[k], next, far)
-                              : diff(true, false, last[0], far, prev, c[k], next);
-      const float gy = diff(by, first[1], last[1], ya[bz], c[2 * bz], c[2 * bz + 1], yb[bz]);
-      const float gz = diff(bz, first[2], last[2], za[by], c[by], c[2 + by], zb[by]);
-      const float gr[3] = {gx * inv2h, gy * inv2h, gz * inv2h};
-      const float m2 = gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2];
-      const float inv = (isfinite(m2) && m2 > 0.f) ? rsqrtf(m2) : 0.f;
-      const float w = fx * (by ? t[1] : 1.f - t[1]) * (bz ? t[2] : 1.f - t[2]);
-      s += w * c[k];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) mv[a] += w * gr[a] * inv;
-    }
-    // lanes 1 and 2 together
-    s += __shfl_xor_sync(kFull, s, 3);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) mv[a] += __shfl_xor_sync(kFull, mv[a], 3);
-    const float m2 = mv[0] * mv[0] + mv[1] * mv[1] + mv[2] * mv[2];
-    const float inv = (m2 > 0.f) ? rsqrtf(m2) : 0.f;
-    // lanes 0 to 2 write the normal, lane 3 the distance
-    const int src = (lane & ~3) + 1;
-    const float o0 = __shfl_sync(kFull, mv[0] * inv, src), o1 = __shfl_sync(kFull, mv[1] * inv, src),
-                o2 = __shfl_sync(kFull, mv[2] * inv, src), o3 = __shfl_sync(kFull, s, src);
-    if (base + (lane >> 2) < m) {
-      if (l == 3)
-        sdf_q[i] = o3;
-      else
-        nrm_q[3 * i + l] = l == 0 ? o0 : l == 1 ? o1 : o2;
+      for (int a = 0; a < 3; ++a) {
+        i0[a] = __shfl_sync(kFull, my_i[a], from);
+        t[a] = __shfl_sync(kFull, my_t[a], from);
+      }
+      query_normal_lanes(i0, t, base + from, base + from < m, n, inv2h, phi, sdf_q, nrm_q);
     }
   }
 }
@@ -771,7 +856,7 @@ QParams qparams(const wgeo_handle* h) {
 int launch_query(wgeo_handle* h, const float* q, int64_t m, float* sdf_q, float* nrm_q, cudaStream_t s) {
   if (m == 0) return WGEO_OK;
   if (nrm_q)
-    query_normal_kernel<<<grid_blocks(4 * m, 256, 152 * 32), 256, 0, s>>>(q, m, qparams(h), h->phi, sdf_q, nrm_q);
+    query_normal_kernel<<<grid_blocks(m, 256, 152 * 32), 256, 0, s>>>(q, m, qparams(h), h->phi, sdf_q, nrm_q);
   else
     query_kernel<<<grid_blocks(m, 256, 152 * 32), 256, 0, s>>>(q, m, qparams(h), h->phi, sdf_q);
   WGEO_LAUNCH_CHECK();

@@ -50,3 +50,52 @@ def test_query_normals_at_the_edges(res, m):
     if m > 1:
         assert torch.equal(got2[1:], got[1:])
     rec.close()
+
+
+@pytest.mark.parametrize("res,m", [(4, 33), (24, 1000), (64, 100_003)])
+def test_query_normals_do_not_depend_on_the_order_of_the_queries(res, m):
+    """Warps whose queries share cache lines take one thread a query, the others
+    four lanes: the same bits either way."""
+    import __graft_entry__ as g
+    g.build()
+    from paper_2609_20964_gb300 import Reconstructor
+    p, n = synth.sphere_cloud(1500, seed=res)
+    rec = Reconstructor(res, len(p))
+    rec.reconstruct(torch.from_numpy(p).cuda(), torch.from_numpy(n).cuda(), BBOX, res)
+    rng = np.random.default_rng(m)
+    q = rng.uniform(-0.1, 1.1, (m, 3)).astype(np.float32)
+    cell = (q * res).astype(int)
+    rows = np.lexsort((q[:, 0], cell[:, 1], cell[:, 2]))
+    sdf, nrm = rec.query(torch.from_numpy(q).cuda())
+    sdf2, nrm2 = rec.query(torch.from_numpy(q[rows]).cuda())
+    at = torch.from_numpy(rows).cuda()
+    assert torch.equal(sdf[at], sdf2) and torch.equal(nrm[at], nrm2)
+    rec.close()
+
+
+def test_queries_on_a_lattice_take_less_time_than_scattered_ones():
+    """2^22 queries in the order of a lattice share their cache lines; four lanes
+    a query there took nearly as long (0.92 of the time) as scattered ones."""
+    import __graft_entry__ as g
+    g.build()
+    from paper_2609_20964_gb300 import Reconstructor
+    p, n = synth.sphere_cloud(20_000, seed=1)
+    rec = Reconstructor(128, len(p))
+    rec.reconstruct(torch.from_numpy(p).cuda(), torch.from_numpy(n).cuda(), BBOX, 128)
+    k = (torch.arange(161, device="cuda") + 0.37) / 161
+    lattice = torch.stack(torch.meshgrid(k, k, k, indexing="ij")[::-1], -1).reshape(-1, 3).contiguous()
+    scattered = lattice[torch.randperm(len(lattice), device="cuda")].contiguous()
+
+    def time(q):
+        ms = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            rec.query(q)
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        return sorted(ms[3:])[4]
+
+    assert time(lattice) <= 0.75 * time(scattered)
+    rec.close()
