@@ -46,3 +46,30 @@ def test_probe_batches_match_the_oracle(kind, n):
     assert np.array_equal(st.cpu().numpy().astype(np.int64), os_)
     assert np.array_equal(out.cpu().numpy(), on)
     rec.close()
+
+
+def test_a_filled_box_takes_no_longer_than_a_surface():
+    """200,000 points that fill a box, every probe beside points, against as many
+    on a sphere: 0.8 of its time; 1.5 with rows taken from the first."""
+    import __graft_entry__ as g
+    g.build()
+    from paper_2609_20964_gb300 import Reconstructor
+    n, times = 200_000, {}
+    rec = Reconstructor(16, n)
+    for kind in ("volume", "sphere"):
+        rng = np.random.default_rng(1)
+        x = _cloud(kind, rng, n)
+        d = x - 0.5 if kind == "sphere" else rng.standard_normal((n, 3))
+        p = torch.from_numpy(x.astype(np.float32)).cuda()
+        N = torch.from_numpy((d / np.linalg.norm(d, axis=1, keepdims=True)).astype(np.float32)).cuda()
+        ms = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            rec.orient_normals(p, N, BOX)
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        times[kind] = sorted(ms[3:])[4]
+    assert times["volume"] <= 1.15 * times["sphere"], times
+    rec.close()
