@@ -2703,10 +2703,15 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
   // stride of the coarsest lattice.  A coarser one costs fewer searches from
   // nothing (4,300 warp instructions a node at 128^3, 7,200 at 256^3), but its
   // patch passes have too few blocks to fill the chip and boxes with many
-  // candidates.  Search stage at 64^3 / 128^3 / 256^3 / 512^3, ms: stride 2
-  // 0.32 / - / - / -, 4 0.37 / 1.70 / 11.8 / 102, 8 0.47 / 2.05 / 11.5 / 85, 16
-  // at 512^3 94.
-  const int coarse = res <= 80 ? 2 : res <= 160 ? 4 : 8;
+  // candidates.  Search stage, us, star body / sphere / small sphere / points
+  // that fill the box: stride 2 against 4 at 72^3 425 447 233 646 / 445 464 181
+  // 734, at 80^3 595 569 325 857 / 587 555 239 929, at 96^3 981 954 577 1265 /
+  // 776 858 397 1176; 4 against 8 at 160^3 2840 3279 1458 4495 / 3055 3781 1404
+  // 5490, at 176^3 3745 4511 1889 5198 / 3907 4965 1831 6115, at 224^3 7744 9110
+  // 4227 12161 / 7603 9827 3946 13069.  Above 160^3 the shape decides, up to 10%
+  // either way (the swimming ellipsoid at 192^3 3.8 / 3.6 ms); at 256^3 11.8 /
+  // 11.5 ms (star body), at 512^3 102 / 85.
+  const int coarse = res < 80 ? 2 : res <= 160 ? 4 : 8;
   rc = node_pass(false, coarse);
   if (rc) return rc;
   for (int stride = coarse / 2; stride >= 1; stride /= 2) {
@@ -2714,9 +2719,12 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
     const int nblk = ((nl + 7) / 8) * ((nl + 7) / 8) * ((nl + 3) / 4);
     // leaves in a block's reach above which its nodes are searched one by one:
     // cheaper in a block (a third of the instructions), but where the blocks
-    // are few the longest decides.  Search stage at 256 / 512 / 1024, ms: 0.29 /
-    // 0.38 / 0.53 on a 64^3 sphere (every triangle is in reach of its centre),
-    // 1.76 / 1.57 / 1.68 at 128^3, 14.2 / 11.5 / 10.8 at 256^3.
+    // are few the longest decides.  Search stage, us, star body / sphere / two
+    // shells / points that fill the box: 256 against 512 at 72^3 423 447 326 642 /
+    // 405 505 328 563, at 88^3 698 717 443 1192 / 670 781 545 993, at 96^3 827 859
+    // 506 1403 / 774 856 611 1170, at 128^3 1708 1919 1075 2997 / 1515 1747 1147
+    // 2367; 512 against kFront at 160^3 (16,000 blocks) 2842 3285 2115 4509 / 2819
+    // 3342 2419 4181, at 176^3 (21,296) 3910 5005 2719 6659 / 3816 4706 3050 6008.
     const int leaf_max = res <= 80 ? 256 : nblk <= 16384 ? 512 : kFront;
     if (ctri) {
       if (count)

@@ -94,3 +94,31 @@ def test_closest_triangles_do_not_depend_on_the_capacities(W):
         rec.close()
         want = want or got
         assert all(torch.equal(a, b) for a, b in zip(got, want)), (max_res, cap)
+
+
+@pytest.mark.parametrize("res", [72, 224])
+def test_search_beside_the_lines_of_the_coarsest_lattice(W, res):
+    test_search_finds_the_nearest_triangle(W, res, 1)
+
+
+@pytest.mark.parametrize("res", [24, 64, 96])
+def test_closest_triangles_at_the_centre_of_a_sphere(W, res):
+    """The nodes that are searched one by one keep a triangle that is nearest to
+    within float32 rounding, the one that their distance belongs to."""
+    bbox = np.array([0, 0, 0, 1, 1, 1], dtype=np.float32)
+    p, n = synth.sphere_cloud(4096, seed=2)
+    rec = W(res, len(p))
+    sdf, _ = rec.reconstruct(_t(p), _t(n), bbox, res, with_normals=False)
+    c = np.arange(res // 2 - 3, res // 2 + 3)
+    lin = ((c[:, None, None] * res + c[None, :, None]) * res + c[None, None, :]).reshape(-1)
+    verts, _ = rec.mesh()
+    tri = verts.astype(np.float64)[rec.field("closest").cpu().numpy().reshape(-1)[lin]]
+    k, j, i = lin // (res * res), lin // res % res, lin % res
+    nodes = (np.stack([i, j, k], 1) + 0.5) / res
+    y, _ = S.closest_point_triangle(nodes, tri[:, 0], tri[:, 1], tri[:, 2])
+    own = np.linalg.norm(nodes - y, axis=1)
+    nearest, _ = S.exact_distance(nodes, verts.astype(np.float64))
+    bound = 4e-7 * nearest + 3e-7      # the distances' of this file
+    assert (own - nearest <= bound).all()
+    assert (np.abs(np.abs(sdf.cpu().numpy().reshape(-1)[lin]) - own) <= bound).all()
+    rec.close()
