@@ -21,9 +21,11 @@
 //
 // Distance: exact minimum over all triangles of the point-to-triangle distance
 // (closest point by Voronoi regions of the triangle: vertices, edges, face —
-// the method of Ericson, Real-Time Collision Detection, 5.1.5), found by a
-// depth-first, nearest-child-first traversal of an implicit octree of brick
-// bounding boxes, pruned only by exact box lower bounds.  Sign: +1 where
+// the method of Ericson, Real-Time Collision Detection, 5.1.5), found through
+// an implicit octree over the bricks whose nodes bound their triangles by
+// fitted solid cylinders (pucks), pruned only by lower bounds of them.  Grid
+// nodes are searched on nested lattices, by blocks of nodes that share a walk;
+// off-grid queries 32 a warp.  Sign: +1 where
 // chi >= c, -1 where chi < c (the marching-cubes surface separates the two node
 // classes, so this is the parity of crossings of any ray from the node).
 #include <math.h>
@@ -1084,11 +1086,11 @@ __device__ __forceinline__ Ff tri_dist2_ff_exact(const Vec3<Ff> p, const float4*
   return rx * rx + ry * ry + rz * rz;
 }
 
-// Octree entries on the traversal stack: level in bits 27..31, node
-// coordinates (< 512 per axis) in bits 0..8 (x), 9..17 (y), 18..26 (z).  The
-// search stacks this word with the node's pyramid index, so that a pop loads
-// the node's puck at once instead of first looking up its level's offset and
-// dimension.
+// Octree entry: level in bits 27..31, node coordinates (< 512 per axis) in bits
+// 0..8 (x), 9..17 (y), 18..26 (z).  sdf_node_kernel stacks this word beside the
+// node's child mask; sdf_query_kernel with the node's pyramid index, so that a
+// pop loads the node's puck at once instead of first looking up its level's
+// offset and dimension; sdf_patch_kernel's fronts hold the coordinates alone.
 __device__ __forceinline__ unsigned pack_node(int lev, int x, int y, int z) {
   return ((unsigned)lev << 27) | ((unsigned)z << 18) | ((unsigned)y << 9) | (unsigned)x;
 }
@@ -1122,10 +1124,10 @@ __device__ __forceinline__ unsigned pack_node(int lev, int x, int y, int z) {
 // testing each popped puck and each triangle for all of them: 0.7 for the
 // seeds, 2 for the block's walk, 1 + 2.5 for the patch's cubes (of 240 in the
 // block's reach, 74 in the patch's and 6.7 in a node's), 3 for 19 triangle
-// tests a node and 2 for its 3 exact ones.  Search stage before -> now, ms:
-// 0.79 -> 0.32 (64^3, 16,384 points), 2.79 -> 1.61 (128^3), 16.4 -> 11.9
-// (256^3), 137 -> 90 (512^3); 1.47 -> 0.30 on a 64^3 sphere, whose centre kept
-// one warp busy for all of it.
+// tests a node and 2 for its 3 exact ones.  Search stage before -> now, ms, of
+// star bodies: 0.79 -> 0.32 (64^3, 16,384 points), 2.79 -> 1.61 (128^3, 100,000),
+// 16.4 -> 11.9 (256^3, 200,000), 137 -> 90 (512^3, 500,000); 1.47 -> 0.30 on a 64^3
+// sphere, whose centre kept one warp busy for all of it.
 
 // What the search reads and writes (device pointers of the handle).
 struct Search {
@@ -2177,15 +2179,24 @@ __global__ void __launch_bounds__(256) normals_kernel(const float* __restrict__ 
 
 // ---- exact signed distance at arbitrary query points (Sec. 2.4, Eqs. 29-34,
 // evaluated off the grid).  Two kernels: the distance search over queries
-// sorted by cell (a warp of 32 neighbouring queries walks the octree as the
-// node search does), then the sign, one thread per query.
+// sorted by cell, then the sign, one thread per query.
 
-// Distance search.  The cut starts from an upper bound: the nearest node's
-// |phi| plus the node's distance to q (triangle inequality), widened for the
-// float rounding of both; with the nodes' closest triangles kept (SEEDS),
-// those of the 8 nodes around q are offered first.  Writes the unsigned distance and the unit
-// direction (q - y) / |q - y| to the closest surface point y (zero when q is
-// on the surface, infinite distance when the mesh is empty).
+// Distance search: a warp of 32 neighbouring queries walks the octree depth
+// first.  A popped node's puck is bounded by every lane against its own query
+// and entered when it beats some lane's cut; children are pushed farthest first
+// by the bound of the warp's first query, and a leaf's triangles are tested by
+// all lanes, each the same (broadcast) triangle against its own query.
+//
+// The cut starts from an upper bound: the nearest node's |phi| plus the node's
+// distance to q (triangle inequality), widened for the float rounding of both;
+// with the nodes' closest triangles kept (SEEDS), those of the 8 nodes around q
+// are offered first.  Writes the unsigned distance and the unit direction (q -
+// y) / |q - y| to the closest surface point y (zero when q is on the surface,
+// infinite distance when the mesh is empty).
+//
+// Bound: instruction issue and latency (10^6 uniform queries at 256^3, 2.61 ms:
+// 1.48 10^9 warp instructions, 62% of the issue slots at 40% occupancy, waits on
+// global loads 4.5 of 11 cycles an instruction; DRAM 1%).
 template <bool SEEDS>
 __global__ void __launch_bounds__(kWarps * 32, 8) sdf_query_kernel(const float* __restrict__ phi, SurfParams g,
                                                                 const Tri* __restrict__ tris,
