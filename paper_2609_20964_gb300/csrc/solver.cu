@@ -916,17 +916,18 @@ __global__ void __launch_bounds__(kSmallThreads) small_vcycle_kernel(float* __re
     float* x = xs + off[L - 1];
     float* b = bsm + off[L - 1];
     // a coarsest level of at most 4^3 below a hierarchy needs only a rough solve
-    if (n <= 4 && L > 1) {
-      small_rbgs(x, b, n, 2 * n + 8, 0);
-    } else {
+    int sweeps = 2 * n + 8;
+    if (n > 4 || L == 1) {
       small_basis(qs, n);
       small_direct(x, b, n, qs, false);
+      sweeps = 0;
       if (shift && L == 1) {   // the whole grid; the solve used b up
         for (int t = threadIdx.x; t < N0; t += blockDim.x) bsm[t] = (bg[t] - sh) - meanb;
         __syncthreads();
-        small_rbgs(x, b, n, kPolish, 0);
+        sweeps = kPolish;
       }
     }
+    if (sweeps) small_rbgs(x, b, n, sweeps, 0);
   }
   // up
   for (int l = L - 2; l >= 0; --l) {
@@ -1048,17 +1049,18 @@ __global__ void __launch_bounds__(kSmallThreads) small_vcycle_q1_kernel(float* _
     const int n = ns[L - 1];
     float* x = xs + off[L - 1];
     float* b = bsm + off[L - 1];
-    if (n <= 4 && L > 1) {
-      small_gs8(x, b, n, 2 * n + 8, 0, 1);
-    } else {
+    int sweeps = 2 * n + 8;
+    if (n > 4 || L == 1) {
       small_basis(qs, n);
       small_direct(x, b, n, qs, true);
+      sweeps = 0;
       if (shift && L == 1) {   // the whole grid; the solve used b up
         for (int t = threadIdx.x; t < N0; t += blockDim.x) bsm[t] = (bg[t] - sh) - meanb;
         __syncthreads();
-        small_gs8(x, b, n, kPolish, 0, 1);
+        sweeps = kPolish;
       }
     }
+    if (sweeps) small_gs8(x, b, n, sweeps, 0, 1);
   }
   for (int l = L - 2; l >= 0; --l) {
     const int n = ns[l], nc = ns[l + 1];
