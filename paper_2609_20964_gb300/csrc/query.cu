@@ -30,6 +30,7 @@ struct QParams {
   int res;
   float lo_hi[3], lo_lo[3];   // lo and 1 / h as float-float pairs (trilinear cells off the FP64 pipe)
   float ih_hi, ih_lo;
+  float sc;                   // box units -> the search records' (search_scale)
 };
 
 __device__ __forceinline__ int64_t lin3(int i, int j, int k, int n) {
@@ -468,9 +469,9 @@ __global__ void sdf_mc_adjoint_kernel(const float* __restrict__ dphi, const int*
         slivers[atomicAdd(nsliver, 1u)] = (int)o;
         continue;
       }
-      float3 ap = make_float3(p.x - r0.x, p.y - r0.y, p.z - r0.z);
+      float3 ap = make_float3(p.x * g.sc - r0.x, p.y * g.sc - r0.y, p.z * g.sc - r0.z);
       if (tris_lo) {
-        const float4 al = tris_lo[t].a;
+        const float3 al = f3(tris_lo[t].a, g.sc);
         ap = make_float3(ap.x - al.x, ap.y - al.y, ap.z - al.z);
       }
       const float d1 = r1.x * ap.x + r1.y * ap.y + r1.z * ap.z;
@@ -585,9 +586,9 @@ __global__ void exact_adjoint_kernel(const float* __restrict__ q, int nq, const 
     const float3 p = make_float3(q[3 * (int64_t)i], q[3 * (int64_t)i + 1], q[3 * (int64_t)i + 2]);
     const float4* rec = tris_s + kTriRec * (int64_t)t;
     const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
-    float3 ap = make_float3(p.x - r0.x, p.y - r0.y, p.z - r0.z);
+    float3 ap = make_float3(p.x * g.sc - r0.x, p.y * g.sc - r0.y, p.z * g.sc - r0.z);
     if (tris_lo) {
-      const float4 al = tris_lo[t].a;
+      const float3 al = f3(tris_lo[t].a, g.sc);
       ap = make_float3(ap.x - al.x, ap.y - al.y, ap.z - al.z);
     }
     const float d1 = r1.x * ap.x + r1.y * ap.y + r1.z * ap.z;
@@ -848,6 +849,7 @@ QParams qparams(const wgeo_handle* h) {
   const double ih = 1.0 / h->h;
   g.ih_hi = (float)ih;
   g.ih_lo = (float)(ih - (double)g.ih_hi);
+  g.sc = search_scale(h->h);
   return g;
 }
 

@@ -191,7 +191,19 @@ struct SurfParams {
   double h;
   int res;
   int nb;        // bricks per axis
+  float sc, us;  // box units -> the search's units (search_scale), and back
 };
+
+SurfParams surf_params(const wgeo_handle* h, int res) {
+  SurfParams g;
+  for (int a = 0; a < 3; ++a) g.lo[a] = h->lo[a];
+  g.h = h->h;
+  g.res = res;
+  g.nb = div_up(res - 1, kBrick);
+  g.sc = search_scale(h->h);
+  g.us = 1.f / g.sc;
+  return g;
+}
 
 __device__ __forceinline__ int64_t lin3(int i, int j, int k, int n) {
   return ((int64_t)k * n + j) * n + i;
@@ -382,13 +394,13 @@ __global__ void mc_count_kernel(const unsigned* __restrict__ bits, SurfParams g,
   }
 }
 
-// The triangle total and its status, and the node coordinates per axis (the
-// distance search reads them instead of forming them in FP64 at every node).
+// The triangle total and its status, and the node coordinates per axis in the
+// search's units (it reads them instead of forming them in FP64 at every node).
 __global__ void mc_total_kernel(const int* __restrict__ brick_off, int nbricks, int64_t cap,
                                 int* __restrict__ leaf_off, DevState* st, SurfParams g, float* __restrict__ axis) {
   for (int t = threadIdx.x; t < 3 * g.res; t += blockDim.x) {
     const int a = t / g.res, i = t - a * g.res;
-    axis[t] = (float)(g.lo[a] + (i + 0.5) * g.h);
+    axis[t] = (float)(g.lo[a] + (i + 0.5) * g.h) * g.sc;
   }
   if (threadIdx.x != 0) return;
   const long long T = brick_off[nbricks];
@@ -635,14 +647,16 @@ constexpr float kPuckAbs = 2e-7f;
 // Search record of a triangle for the distance search: vertex a and the edge
 // vectors ab, ac with the Gram entries |ab|^2, ab.ac and |ac|^2, and the
 // reciprocals the Voronoi regions divide by (0 for a zero-length edge or a
-// collapsed triangle).
+// collapsed triangle), all in the search's units (sc).
 // With the vertices' low parts (lo, may be null) the edge vectors are the
 // float32 roundings of the differences of the ~48-bit vertices, not the
 // differences of the float32 vertices: their directions then carry float32
 // rounding (~6e-8 relative) instead of the vertices' absolute rounding,
 // which a far node's closest point would amplify by distance / edge length.
-__device__ __forceinline__ void write_search_record(const Tri& tr, const Tri* lo, float4* __restrict__ rec) {
-  const float3 a = f3(tr.a), b = f3(tr.b), c = f3(tr.c);
+__device__ __forceinline__ void write_search_record(const Tri& tr, const Tri* lo, float sc,
+                                                    float4* __restrict__ rec) {
+  float3 a = f3(tr.a);
+  const float3 b = f3(tr.b), c = f3(tr.c);
   float3 ab = sub3(b, a), ac = sub3(c, a), bc = sub3(c, b);
   if (lo) {
     const float3 al = f3(lo->a), bl = f3(lo->b), cl = f3(lo->c);
@@ -650,6 +664,10 @@ __device__ __forceinline__ void write_search_record(const Tri& tr, const Tri* lo
     ac = make_float3(ac.x + (cl.x - al.x), ac.y + (cl.y - al.y), ac.z + (cl.z - al.z));
     bc = make_float3(bc.x + (cl.x - bl.x), bc.y + (cl.y - bl.y), bc.z + (cl.z - bl.z));
   }
+  a = make_float3(a.x * sc, a.y * sc, a.z * sc);
+  ab = make_float3(ab.x * sc, ab.y * sc, ab.z * sc);
+  ac = make_float3(ac.x * sc, ac.y * sc, ac.z * sc);
+  bc = make_float3(bc.x * sc, bc.y * sc, bc.z * sc);
   const float e00 = dot3(ab, ab), e11 = dot3(ac, ac), ebc = dot3(bc, bc);
   const float3 cr = cross3(ab, ac);
   const float det = dot3(cr, cr);   // = |ab|^2 |ac|^2 - (ab.ac)^2, without the cancellation
@@ -692,11 +710,23 @@ __global__ void puck_leaf_scan_kernel(const int* __restrict__ leaf_off, int nb, 
   }
 }
 
-// Puck (centre + radius, axis + half-thickness) fitted to the vertices of
-// triangles [q0, q1): centroid and mean area normal, then the largest radial
+// v / |v|, (0, 0, 1) for no direction, by way of a power of two that brings v's
+// largest component near 1: a sum of area normals is a square of the box's
+// units, and its square can leave the float range.
+__device__ __forceinline__ float3 unit_normal(float3 v) {
+  const unsigned e = __float_as_uint(fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fabsf(v.z))) >> 23;
+  const float k = __uint_as_float((254u - min(e, 253u)) << 23);
+  v = make_float3(v.x * k, v.y * k, v.z * k);
+  const float nn = sqrtf(dot3(v, v));
+  return nn > 0.f ? make_float3(v.x / nn, v.y / nn, v.z / nn) : make_float3(0.f, 0.f, 1.f);
+}
+
+// Puck (centre + radius, axis + half-thickness, in the search's units) fitted to
+// the vertices of triangles [q0, q1): centroid and mean area normal, then the largest radial
 // and axial vertex offsets in that frame, padded so the bound stays
 // conservative under float rounding.
-__device__ __forceinline__ void fit_puck(const Tri* __restrict__ tris, int64_t q0, int64_t q1, float4& A, float4& B) {
+__device__ __forceinline__ void fit_puck(const Tri* __restrict__ tris, int64_t q0, int64_t q1, float sc, float4& A,
+                                         float4& B) {
   float3 cs = make_float3(0.f, 0.f, 0.f), ns = make_float3(0.f, 0.f, 0.f);
   for (int64_t q = q0; q < q1; ++q) {
     const Tri tr = tris[q];
@@ -711,8 +741,7 @@ __device__ __forceinline__ void fit_puck(const Tri* __restrict__ tris, int64_t q
   }
   const float inv = 1.f / (3.f * (float)(q1 - q0));
   const float3 cc = make_float3(cs.x * inv, cs.y * inv, cs.z * inv);
-  const float nn = sqrtf(dot3(ns, ns));
-  const float3 nv = nn > 0.f ? make_float3(ns.x / nn, ns.y / nn, ns.z / nn) : make_float3(0.f, 0.f, 1.f);
+  const float3 nv = unit_normal(ns);
   float r = 0.f, th = 0.f;
   for (int64_t q = q0; q < q1; ++q) {
     const Tri tr = tris[q];
@@ -727,8 +756,8 @@ __device__ __forceinline__ void fit_puck(const Tri* __restrict__ tris, int64_t q
     }
   }
   const float pad = kPuckRel * (r + th) + kPuckAbs * (fabsf(cc.x) + fabsf(cc.y) + fabsf(cc.z));
-  A = make_float4(cc.x, cc.y, cc.z, r + pad);
-  B = make_float4(nv.x, nv.y, nv.z, th + pad);
+  A = make_float4(cc.x * sc, cc.y * sc, cc.z * sc, (r + pad) * sc);
+  B = make_float4(nv.x, nv.y, nv.z, (th + pad) * sc);
 }
 
 // Rank of the q-th triangle of a leaf in a depth-first walk of the octree that
@@ -754,7 +783,7 @@ __global__ void puck_leaf_kernel(const Tri* __restrict__ tris, Tri* __restrict__
                                  const int* __restrict__ leaf_off, const unsigned* __restrict__ leaf_cnt, int nb,
                                  int64_t cap, const int* __restrict__ live, const DevState* __restrict__ st,
                                  float4* __restrict__ pyr, float4* __restrict__ tris_s,
-                                 float4* __restrict__ cell_pyr) {
+                                 float4* __restrict__ cell_pyr, float sc) {
   const int nl = 2 * nb;
   const int64_t nlive = st->nleaf_live;
   for (int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; it < nlive;
@@ -768,14 +797,14 @@ __global__ void puck_leaf_kernel(const Tri* __restrict__ tris, Tri* __restrict__
       const Tri tr = tris[q];
       if (tris_lo) {
         const Tri tl = tris_lo[q];
-        write_search_record(tr, &tl, tris_s + kTriRec * q);
+        write_search_record(tr, &tl, sc, tris_s + kTriRec * q);
         tris_lo[q].a.w = __uint_as_float(walk_rank(lx, ly, lz, (int)(q - s0)));
       } else {
-        write_search_record(tr, nullptr, tris_s + kTriRec * q);
+        write_search_record(tr, nullptr, sc, tris_s + kTriRec * q);
       }
     }
     float4 A, B;
-    fit_puck(tris, s0, s1, A, B);
+    fit_puck(tris, s0, s1, sc, A, B);
     pyr[2 * t] = A;
     pyr[2 * t + 1] = B;
     if (cell_pyr) {
@@ -784,7 +813,7 @@ __global__ void puck_leaf_kernel(const Tri* __restrict__ tris, Tri* __restrict__
       for (; cn != 0u; cn >>= 4) {
         const int64_t q1 = min(q0 + (int64_t)(cn & 15u), s1);
         if (q0 < q1) {
-          fit_puck(tris, q0, q1, A, B);
+          fit_puck(tris, q0, q1, sc, A, B);
           cell_pyr[2 * q0] = A;
           cell_pyr[2 * q0 + 1] = B;
         }
@@ -815,7 +844,8 @@ __device__ __forceinline__ float puck_dist2(const float3 p, const float4 A, cons
 }
 
 // Vertex-fitted pucks for every octree level above the leaves.  A node's
-// frame is its vertex centroid and mean area normal; both come from sums
+// frame is its vertex centroid and mean area normal (in the box's units; the
+// finished pucks are brought to the search's); both come from sums
 // that add up the tree (per brick first: a level-1 node is one brick).  The
 // radius and half-thickness are the largest radial and axial vertex offsets
 // in that frame, taken in one pass over the leaves for all levels at once
@@ -824,8 +854,7 @@ __device__ __forceinline__ float puck_dist2(const float3 p, const float4 A, cons
 __device__ __forceinline__ void node_frame(const float4 s0, const float4 s1, float3& c, float3& ax) {
   const float inv = 1.f / (3.f * s0.w);
   c = make_float3(s0.x * inv, s0.y * inv, s0.z * inv);
-  const float nn = sqrtf(s1.x * s1.x + s1.y * s1.y + s1.z * s1.z);
-  ax = nn > 0.f ? make_float3(s1.x / nn, s1.y / nn, s1.z / nn) : make_float3(0.f, 0.f, 1.f);
+  ax = unit_normal(f3(s1));
 }
 
 __global__ void puck_sums_brick_kernel(const Tri* __restrict__ tris, const int* __restrict__ brick_off, int nb,
@@ -930,7 +959,7 @@ __global__ void puck_rth_kernel(const Tri* __restrict__ tris, const int* __restr
 }
 
 __global__ void puck_finalize_kernel(float4* __restrict__ pyr, const float4* __restrict__ sums,
-                                     const unsigned* __restrict__ rth, int64_t naux, int64_t pyr_base) {
+                                     const unsigned* __restrict__ rth, int64_t naux, int64_t pyr_base, float sc) {
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < naux; a += (int64_t)gridDim.x * blockDim.x) {
     const float4 s0 = sums[2 * a], s1 = sums[2 * a + 1];
     const int64_t gi = pyr_base + a;
@@ -943,8 +972,8 @@ __global__ void puck_finalize_kernel(float4* __restrict__ pyr, const float4* __r
     node_frame(s0, s1, c, ax);
     const float r = __uint_as_float(rth[2 * a]), th = __uint_as_float(rth[2 * a + 1]);
     const float pad = kPuckRel * (r + th) + kPuckAbs * (fabsf(c.x) + fabsf(c.y) + fabsf(c.z));
-    pyr[2 * gi] = make_float4(c.x, c.y, c.z, r + pad);
-    pyr[2 * gi + 1] = make_float4(ax.x, ax.y, ax.z, th + pad);
+    pyr[2 * gi] = make_float4(c.x * sc, c.y * sc, c.z * sc, (r + pad) * sc);
+    pyr[2 * gi + 1] = make_float4(ax.x, ax.y, ax.z, (th + pad) * sc);
   }
 }
 
@@ -1066,13 +1095,13 @@ __device__ __forceinline__ unsigned feature_class(float v, float w, const Tri* _
 // and rounding of the weights, change |p - y| only to second order (the
 // residual is normal to the directions they move y in).
 __device__ __forceinline__ Ff tri_dist2_ff_exact(const Vec3<Ff> p, const float4* __restrict__ rec, const Tri& hi,
-                                                 const Tri& lo) {
+                                                 const Tri& lo, float sc) {
   const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3];
-  const Ff ax = Ff(hi.a.x) + Ff(lo.a.x), ay = Ff(hi.a.y) + Ff(lo.a.y), az = Ff(hi.a.z) + Ff(lo.a.z);
-  const Ff abx = (Ff(hi.b.x) + Ff(lo.b.x)) - ax, aby = (Ff(hi.b.y) + Ff(lo.b.y)) - ay,
-           abz = (Ff(hi.b.z) + Ff(lo.b.z)) - az;
-  const Ff acx = (Ff(hi.c.x) + Ff(lo.c.x)) - ax, acy = (Ff(hi.c.y) + Ff(lo.c.y)) - ay,
-           acz = (Ff(hi.c.z) + Ff(lo.c.z)) - az;
+  const float3 ah = f3(hi.a, sc), bh = f3(hi.b, sc), ch = f3(hi.c, sc);
+  const float3 al = f3(lo.a, sc), bl = f3(lo.b, sc), cl = f3(lo.c, sc);
+  const Ff ax = Ff(ah.x) + Ff(al.x), ay = Ff(ah.y) + Ff(al.y), az = Ff(ah.z) + Ff(al.z);
+  const Ff abx = (Ff(bh.x) + Ff(bl.x)) - ax, aby = (Ff(bh.y) + Ff(bl.y)) - ay, abz = (Ff(bh.z) + Ff(bl.z)) - az;
+  const Ff acx = (Ff(ch.x) + Ff(cl.x)) - ax, acy = (Ff(ch.y) + Ff(cl.y)) - ay, acz = (Ff(ch.z) + Ff(cl.z)) - az;
   const Ff apx = p.x - ax, apy = p.y - ay, apz = p.z - az;
   const float3 ap = make_float3(apx.hi, apy.hi, apz.hi);
   const float d1 = r1.x * ap.x + r1.y * ap.y + r1.z * ap.z;
@@ -1144,8 +1173,9 @@ struct Search {
   int64_t cap;
   int n;                    // nodes per axis
   int nb;                   // bricks per axis
-  float h;
-  float coord;              // largest |coordinate| of the box
+  float h;                  // cell size and
+  float coord;              // largest |coordinate| of the box, in the search's units
+  float sc, us;             // box units -> the search's, and back
   float* phi;
   float* sdf_out;
   int* ctri;
@@ -1270,7 +1300,7 @@ __device__ __forceinline__ void store_nodes(const Search& S, const Cands<TIES>& 
   }
   if (!valid) return;
   const int bt = c.ct[0];
-  const float val = (S.chi[o] >= S.st->c_up ? 1.f : -1.f) * sqrtf(c.cd[0]);
+  const float val = (S.chi[o] >= S.st->c_up ? 1.f : -1.f) * sqrtf(c.cd[0]) * S.us;
   S.phi[o] = val;
   if (S.sdf_out) S.sdf_out[o] = val;
   if (S.ctri) S.ctri[o] = bt;
@@ -2056,7 +2086,7 @@ __global__ void sdf_tie_kernel(const __grid_constant__ Search S, SurfParams g, i
   const int n = g.res;
   for (int t = threadIdx.x; t < 3 * n; t += blockDim.x) {
     const int a = t / n, i = t % n;
-    const double v = g.lo[a] + (i + 0.5) * g.h;
+    const double v = (g.lo[a] + (i + 0.5) * g.h) * (double)g.sc;
     const float hi = (float)v;
     s_ax[a][i] = make_float2(hi, (float)(v - (double)hi));
   }
@@ -2111,7 +2141,8 @@ __global__ void sdf_tie_kernel(const __grid_constant__ Search S, SurfParams g, i
         bi = cand[q];
         break;
       }
-      const Ff d2 = tri_dist2_ff_exact(pf, S.tris_s + kTriRec * (int64_t)cand[q], S.tris[cand[q]], S.tris_lo[cand[q]]);
+      const Ff d2 = tri_dist2_ff_exact(pf, S.tris_s + kTriRec * (int64_t)cand[q], S.tris[cand[q]], S.tris_lo[cand[q]],
+                                       S.sc);
       if (bi < 0 || d2 < bd || (!(bd < d2) && cand[q] < bi)) {
         bd = d2;
         bi = cand[q];
@@ -2120,7 +2151,7 @@ __global__ void sdf_tie_kernel(const __grid_constant__ Search S, SurfParams g, i
     S.ctri[o] = bi;
     if (left == 1) continue;
     const float sgn = (S.chi[o] >= cf) ? 1.f : -1.f;
-    const float val = sgn * sqrtf(__fadd_rn(bd.hi, bd.lo));
+    const float val = sgn * sqrtf(__fadd_rn(bd.hi, bd.lo)) * S.us;
     S.phi[o] = val;
     if (S.sdf_out) S.sdf_out[o] = val;
   }
@@ -2224,6 +2255,7 @@ __global__ void __launch_bounds__(kWarps * 32, 8) sdf_query_kernel(const float* 
 #pragma unroll
   for (int a = 0; a < 3; ++a)
     coord = fmaxf(coord, (float)fmax(fabs(g.lo[a]), fabs(g.lo[a] + n * g.h)));
+  coord *= g.sc;
   const int top = pi.nlev - 1;
   const int nb = (s_dim[0] + 1) / 2;
   uint2* stk = s_node[w];
@@ -2232,7 +2264,7 @@ __global__ void __launch_bounds__(kWarps * 32, 8) sdf_query_kernel(const float* 
     const int k = base + lane;
     const bool valid = k < m;
     const float4 e = sorted[valid ? k : base];
-    const float3 p = make_float3(e.x, e.y, e.z);
+    const float3 p = f3(e, g.sc);
     // nearest node and the bound |phi(node)| + |q - node|
     int ni[3];
     const float pq[3] = {e.x, e.y, e.z};
@@ -2242,10 +2274,11 @@ __global__ void __launch_bounds__(kWarps * 32, 8) sdf_query_kernel(const float* 
       ni[a] = (int)fmin(fmax(rint(f), 0.0), (double)(n - 1));
     }
     const int64_t o = lin3(ni[0], ni[1], ni[2], n);
-    const float3 nd = make_float3((float)(g.lo[0] + (ni[0] + 0.5) * g.h), (float)(g.lo[1] + (ni[1] + 0.5) * g.h),
-                                  (float)(g.lo[2] + (ni[2] + 0.5) * g.h));
+    const float3 nd = make_float3((float)(g.lo[0] + (ni[0] + 0.5) * g.h) * g.sc,
+                                  (float)(g.lo[1] + (ni[1] + 0.5) * g.h) * g.sc,
+                                  (float)(g.lo[2] + (ni[2] + 0.5) * g.h) * g.sc);
     const float dn = sqrtf((p.x - nd.x) * (p.x - nd.x) + (p.y - nd.y) * (p.y - nd.y) + (p.z - nd.z) * (p.z - nd.z));
-    const float bnd = (fabsf(phi[o]) + dn) * (1.f + 1e-5f) + 1e-6f * coord;
+    const float bnd = (fabsf(phi[o]) * g.sc + dn) * (1.f + 1e-5f) + 1e-6f * coord;
     float cut = valid ? bnd * bnd : -INFINITY;
     float cd = INFINITY;
     int ct = -1;
@@ -2339,14 +2372,14 @@ __global__ void __launch_bounds__(kWarps * 32, 8) sdf_query_kernel(const float* 
       if (!(r0.w * r2.w * r3.w < kSliverKappa)) {
         // a sliver: the closest point's direction in FP64
         const Tri tr = tris[ct];
-        const double pd[3] = {p.x, p.y, p.z}, ad[3] = {tr.a.x, tr.a.y, tr.a.z}, bd[3] = {tr.b.x, tr.b.y, tr.b.z},
+        const double pd[3] = {e.x, e.y, e.z}, ad[3] = {tr.a.x, tr.a.y, tr.a.z}, bd[3] = {tr.b.x, tr.b.y, tr.b.z},
                      cdv[3] = {tr.c.x, tr.c.y, tr.c.z};
         double bw64[3], dir64[3];
         closest_point_fp64(pd, ad, bd, cdv, bw64, dir64);
         dir = make_float3((float)dir64[0], (float)dir64[1], (float)dir64[2]);
       }
     }
-    dist_out[idx] = ct >= 0 ? sqrtf(cd) : INFINITY;
+    dist_out[idx] = ct >= 0 ? sqrtf(cd) * g.us : INFINITY;
     if (tri_out) tri_out[idx] = ct;
     if (dir_out) {
       dir_out[3 * (int64_t)idx] = dir.x;
@@ -2565,11 +2598,7 @@ size_t pyramid_aux_nodes(int nb) {
 }
 
 int launch_isovalue(wgeo_handle* h, const float* points, int64_t n, int res, cudaStream_t s) {
-  SurfParams g;
-  for (int a = 0; a < 3; ++a) g.lo[a] = h->lo[a];
-  g.h = h->h;
-  g.res = res;
-  g.nb = div_up(res - 1, kBrick);
+  const SurfParams g = surf_params(h, res);
   const int nbk = grid_blocks(n, 256, kPartials);
   if (n > 0) {
     isovalue_kernel<<<nbk, 256, 0, s>>>(points, n, h->pcell, h->chi32, g, h->partials);
@@ -2583,11 +2612,7 @@ int launch_isovalue(wgeo_handle* h, const float* points, int64_t n, int res, cud
 }
 
 int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_out, cudaStream_t s) {
-  SurfParams g;
-  for (int a = 0; a < 3; ++a) g.lo[a] = h->lo[a];
-  g.h = h->h;
-  g.res = res;
-  g.nb = div_up(res - 1, kBrick);
+  const SurfParams g = surf_params(h, res);
   const int nbricks = g.nb * g.nb * g.nb;
   int slot = stage_begin(h, kStMC, s);
   {
@@ -2628,7 +2653,7 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
   WGEO_LAUNCH_CHECK();
   const int live_grid = grid_blocks(nleaf, 256, h->num_sms * 8);
   puck_leaf_kernel<<<live_grid, 256, 0, s>>>(h->tris, h->tris_lo, h->leaf_off, h->leaf_cnt, g.nb, h->mesh_cap, live,
-                                             h->dstate, h->pyramid, h->tris_s, h->cell_pyr);
+                                             h->dstate, h->pyramid, h->tris_s, h->cell_pyr, g.sc);
   WGEO_LAUNCH_CHECK();
   {
     // levels >= 1: sums per brick, sums up the tree, vertex maxima, pucks
@@ -2647,7 +2672,7 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
     WGEO_LAUNCH_CHECK();
     const int64_t naux = pi.off[pi.nlev - 1] + 1 - pi.off[1];
     puck_finalize_kernel<<<grid_blocks(naux, 256, 152 * 16), 256, 0, s>>>(h->pyramid, h->pyr_sums, h->pyr_rth,
-                                                                          naux, pi.off[1]);
+                                                                          naux, pi.off[1], g.sc);
     WGEO_LAUNCH_CHECK();
     puck_mask_kernel<<<grid_blocks(naux, 256, 152 * 16), 256, 0, s>>>(h->pyramid, pi);
     WGEO_LAUNCH_CHECK();
@@ -2675,10 +2700,13 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
   S.cap = h->mesh_cap;
   S.n = res;
   S.nb = g.nb;
-  S.h = (float)g.h;
+  S.h = (float)g.h * g.sc;
   S.coord = 0.f;
   for (int a = 0; a < 3; ++a)
     S.coord = std::max(S.coord, (float)std::max(fabs(g.lo[a]), fabs(g.lo[a] + res * g.h)));
+  S.coord *= g.sc;
+  S.sc = g.sc;
+  S.us = g.us;
   S.phi = h->phi;
   S.sdf_out = sdf_out;
   S.ctri = ctri;
@@ -2778,11 +2806,7 @@ int launch_mc_sdf_normals(wgeo_handle* h, int res, float* sdf_out, float* nrm_ou
 int launch_query_exact_chunk(wgeo_handle* h, const float* q, int nq, float* sdf_q, float* nrm_q, int* tri,
                              cudaStream_t s) {
   if (nq == 0) return WGEO_OK;
-  SurfParams g;
-  for (int a = 0; a < 3; ++a) g.lo[a] = h->lo[a];
-  g.h = h->h;
-  g.res = h->res;
-  g.nb = div_up(h->res - 1, kBrick);
+  const SurfParams g = surf_params(h, h->res);
   const PyrInfo pi = pyramid_info(2 * g.nb);
   const int* ctri = h->opt.keep_for_backward ? h->ctri : nullptr;
   // queries sorted by (cell of 8 h, sub-cell key), so that a warp's 32

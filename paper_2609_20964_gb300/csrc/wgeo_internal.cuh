@@ -212,6 +212,7 @@ __device__ __forceinline__ float2 split_f64(double v) {
 }
 
 __device__ __forceinline__ float3 f3(const float4 v) { return make_float3(v.x, v.y, v.z); }
+__device__ __forceinline__ float3 f3(const float4 v, float s) { return make_float3(v.x * s, v.y * s, v.z * s); }
 __device__ __forceinline__ float3 sub3(float3 a, float3 b) { return make_float3(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 
@@ -245,9 +246,23 @@ __device__ __forceinline__ bool operator>(Ff a, Ff b) { return b < a; }
 __device__ __forceinline__ bool operator<=(Ff a, Ff b) { return !(b < a); }
 __device__ __forceinline__ bool operator>=(Ff a, Ff b) { return !(a < b); }
 
+// Power of two that brings the cell size into [1, 2).  The distance search works
+// in these units (search records, pucks, node positions and the points tested
+// against them), so that its fourth powers of a length, and their reciprocals
+// on thin triangles, neither overflow nor underflow whatever the box's units:
+// in the box's own, 1 / |ab x ac|^2 overflows on thin triangles of a 10^-6 box.
+// Scaling by a power of two is exact, so results are the same bits in any units.
+inline float search_scale(double h) {
+  int e;
+  frexp(h, &e);   // h = m 2^e, m in [1/2, 1)
+  const int k = 1 - e;
+  return ldexpf(1.f, k < -126 ? -126 : k > 126 ? 126 : k);
+}
+
 // Closest-point weights (v, w) of y = a + v ab + w ac on a triangle given by
 // its search record (r0 = (a, |ab|^2), r1 = (ab, ab.ac), r2 = (ac, |ac|^2),
-// r3 = (1/|ab|^2, 1/|ac|^2, 1/|bc|^2, 1/|ab x ac|^2)), from ap = p - a,
+// r3 = (1/|ab|^2, 1/|ac|^2, 1/|bc|^2, 1/|ab x ac|^2)), from ap = p - a (in the
+// record's units),
 // d1 = ab.ap and d2 = ac.ap: Ericson's Voronoi-region case analysis with the
 // six dot products reduced to two through the Gram entries and the
 // divisions replaced by the reciprocals.

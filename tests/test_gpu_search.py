@@ -122,3 +122,23 @@ def test_closest_triangles_at_the_centre_of_a_sphere(W, res):
     assert (own - nearest <= bound).all()
     assert (np.abs(np.abs(sdf.cpu().numpy().reshape(-1)[lin]) - own) <= bound).all()
     rec.close()
+
+
+@pytest.mark.parametrize("keep", [1, 0])
+@pytest.mark.parametrize("res", [20, 64, 256])
+def test_distances_scale_with_the_units_of_the_box(W, res, keep):
+    """A box of 2^k gives 2^k times the distances of the unit box, whatever its
+    units: scaling by a power of two is exact, and the search's fourth powers of
+    a length do not leave the float range."""
+    p, n = synth.sphere_cloud(3000, seed=7)
+    q = np.random.default_rng(3).uniform(0, 1, (500, 3)).astype(np.float32)
+    rec = W(res, len(p), keep_for_backward=keep)
+    want = None
+    for k in (0, -20, -24, -30, -40, 40):
+        s = np.float32(2.0) ** k
+        sdf, nrm = rec.reconstruct(_t(p * s), _t(n), np.array([0, 0, 0, s, s, s], np.float32), res)
+        got = [sdf / float(s), nrm, rec.query_exact(_t(q * s), with_grad=False)[0] / float(s)]
+        want = want or got
+        for a, b in zip(got, want):
+            assert bool(torch.isfinite(a).all()) and float((a - b).norm() / b.norm()) <= 1e-6, k
+    rec.close()
