@@ -430,7 +430,7 @@ struct wgeo_handle {
   int* tile_off = nullptr;       // ntiles + 1
   int* tile_cursor = nullptr;
 
-  float* axis = nullptr;         // node coordinates of the last forward, [3][res]
+  float* axis = nullptr;         // node coordinates of the last forward, [3][res], in the search's units
 
   // mesh
   int64_t mesh_cap = 0;
@@ -442,7 +442,8 @@ struct wgeo_handle {
   wgeo::Tri* tris_lo = nullptr;  // keep_for_backward: per vertex the low part of its ~48-bit position
                                  // (FP64 vertex - float32 vertex); null otherwise
   float4* tris_s = nullptr;      // per triangle: search record (a, |ab|^2), (ab, ab.ac), (ac, |ac|^2),
-                                 // (1/|ab|^2, 1/|ac|^2, 1/|bc|^2, 1/|ab x ac|^2)
+                                 // (1/|ab|^2, 1/|ac|^2, 1/|bc|^2, 1/|ab x ac|^2); like the pucks in
+                                 // the search's units (search_scale)
   float4* pyramid = nullptr;     // 2 float4 per node (puck: centre + radius, axis + half-thickness)
   float4* cell_pyr = nullptr;    // per cube with triangles: its puck, at the slot of its first triangle
   float4* pyr_sums = nullptr;    // levels >= 1: vertex sum + count, area-normal sum (puck construction)
